@@ -6,6 +6,7 @@
 #include <new>
 
 #include "fem_internal.h"
+#include "fx_layout.h"
 
 namespace {
 
@@ -260,7 +261,8 @@ int fem_wait_timeouts(unsigned long long *count, int reset) {
 
 int fem_layout_check(int64_t *violations) {
     if (!violations) return FEM_EINVAL;
-    *violations = (int64_t)fem::layout_violations_bp30() + (int64_t)fem::layout_violations_bp35();
+    *violations = (int64_t)fem::layout_violations_bp30() + (int64_t)fem::layout_violations_bp35() +
+                  (int64_t)fem::fx_table_violations();
     return FEM_OK;
 }
 

@@ -17,6 +17,7 @@
 // (bp35_point.cuh, Algorithm 7)) is chosen by a small autotuner that times
 // every candidate on the batch itself; the chosen configuration can be
 // replayed from a CUDA graph that contains the counter reset and the kernel.
+#define FEM_FX_TABLES
 #include <algorithm>
 #include <cstring>
 #include <new>
@@ -24,7 +25,7 @@
 
 #include "bp30_body.cuh"
 #include "bp30_point.cuh"
-#include "bp35_body.cuh"
+#include "bp35_fx.cuh"
 #include "bp35_point.cuh"
 
 namespace fem {
@@ -69,7 +70,7 @@ struct Epb30 {
 
 template <int THREADS, int N>
 constexpr int batch_smem_n() {
-    constexpr int s35 = Bp35Layout<double, N, Epb35<THREADS, N>::v>::smem;
+    constexpr int s35 = Fx35Layout<N, Epb35<THREADS, N>::v>::smem;
     constexpr int s30 = Bp30Layout<N, Epb30<THREADS, N>::v>::smem;
     constexpr int sp = N <= kBatchMaxPointN ? Bp30Point<N>::smem : 0;
     constexpr int sp35 = N <= kBatchMaxPointN35 ? Bp35Point<N>::smem : 0;
@@ -109,8 +110,8 @@ int epb_for(int op, int N) {
 // that each body gets its own register allocation.
 template <int THREADS, int K>
 __device__ __noinline__ void task35(unsigned char *smem, const BatchTask tk, const BatchMesh M) {
-    bp35_block<double, K, Epb35<THREADS, K>::v, false>(smem, tk.e0, tk.nel, M.G, M.lambda, M.q, M.out, nullptr,
-                                                       nullptr, nullptr, nullptr);
+    bp35_fx_block<K, Epb35<THREADS, K>::v, false>(smem, tk.e0, tk.nel, M.G, M.lambda, M.q, M.out, nullptr, nullptr,
+                                                  nullptr, nullptr);
 }
 template <int THREADS, int K>
 __device__ __noinline__ void task30(unsigned char *smem, const BatchTask tk, const BatchMesh M) {
@@ -173,7 +174,7 @@ batch_kernel(const BatchMesh *__restrict__ meshes, const BatchTask *__restrict__
     }
 }
 
-FEM_DEFINE_FOLD_UPLOAD(upload_fold_batch_tu)
+FEM_DEFINE_FX_UPLOAD(upload_fold_batch_tu)
 
 // FP64 instructions per element (even-odd lines; used to order tasks).
 double cost_per_element(int op, int N) {

@@ -1,28 +1,20 @@
-// BP3.5 collocated screened-Poisson matvec (Algorithm 4):
+// FP32 BP3.5 kernels (Algorithm 4), the inner operator of the mixed-precision
+// solver:
 //   Aq = D_r^T Rr + D_s^T Rs + D_t^T Rt + lambda wJ q,
 //   [Rr Rs Rt] = G [q_r q_s q_t],  q_r = (D x I x I) q, ...
-// in IEEE FP64 (the operator of the paper) and in FP32 (the inner operator
-// of the mixed-precision solver), plus a variant fused with the PCG
-// direction update p <- z + beta p and the p . Ap reduction.
+// and the variant fused with the PCG direction update p <- z + beta p and the
+// p . Ap reduction.  The FP64 operator is in bp35_fx.cu.
 //
-// GB300 design.  FP64 issues at 2 instructions per clock per SM on this
-// part (1/64 of the FP32 rate), so the FP64 kernel is bound by its FP64
-// instruction count, not by HBM or shared memory (ncu: FP64 pipe 83-96 %
-// busy, DRAM 4-11 %); the same code in FP32 is bound by HBM.  The design
-// minimises FP64 instructions and spends shared memory, registers and
-// integer issue freely:
+// GB300 design (bp35_body.cuh), bound by HBM:
 //   * every one-dimensional contraction is one thread applying the even-odd
-//     folded D or D^T to a whole line (eo.cuh): about n/2 + 2 instructions
-//     per node instead of n, operator entries as constant-bank operands;
+//     folded D or D^T to a whole line (eo.cuh), operator entries as
+//     constant-bank operands;
 //   * q^e and the r and s partial results of the element live in shared
 //     memory (padded boxes), the t-direction work of a thread's (i, j)
 //     column stays in registers, four barriers per element;
 //   * several elements per block (n^2 threads each), coalesced loads of q
-//     and of each geometric-factor plane, coalesced stores.
-// FP32 at degree up to 9 (the mixed solver's hot kernel) runs as a
-// persistent, double-buffered TMA stream instead (see bp35_stream_kernel),
-// and above 9 as the stream kernel with one factor stage
-// (bp35_stream1_kernel).
+//     and of each geometric-factor plane, coalesced stores;
+//   * where it measured faster, a persistent TMA stream (bp35_stream.cuh).
 #include "bp35_stream.cuh"
 
 namespace fem {
@@ -65,18 +57,6 @@ constexpr auto bp35_fn() {
 }
 
 template <int N>
-struct Bp35Launch {
-    static cudaError_t run(int64_t E, const double *G, double lambda, const double *q, double *Aq,
-                           cudaStream_t s) {
-        using C = Bp35Cfg<double, N>;
-        const int64_t blocks = (E + C::EPB - 1) / C::EPB;
-        bp35_fn<double, N, false>()<<<(unsigned)blocks, C::threads, C::smem, s>>>(
-            E, G, lambda, q, Aq, nullptr, nullptr, nullptr, nullptr);
-        return cudaGetLastError();
-    }
-};
-
-template <int N>
 struct Bp35F32Launch {
     static cudaError_t run(int64_t E, const float *G, double lambda, const float *q, float *Aq,
                            cudaStream_t s) {
@@ -94,35 +74,28 @@ struct Bp35F32Launch {
     }
 };
 
-template <typename T>
-struct Bp35PcgLaunchT {
-    template <int N>
-    struct L {
-        static cudaError_t run(int64_t E, const T *G, double lambda, const T *z, T *p, const double *beta,
-                               T *Ap, double *partials, cudaStream_t s, double *status) {
-            if constexpr (sizeof(T) == 4 && bp35_streamed<N, true, float>()) {
-                return launch_stream35<N, true>(E, G, lambda, nullptr, Ap, z, p, beta, partials, s, nullptr,
-                                                status);
-            } else if constexpr (sizeof(T) == 4 && bp35_streamed1<N, true, float>()) {
-                return launch_stream35_1<N, true>(E, G, lambda, nullptr, Ap, z, p, beta, partials, s, nullptr,
-                                                  status);
-            } else {
-                using C = Bp35Cfg<T, N>;
-                const int64_t blocks = (E + C::EPB - 1) / C::EPB;
-                bp35_fn<T, N, true>()<<<(unsigned)blocks, C::threads, C::smem, s>>>(E, G, lambda, nullptr, Ap, z,
-                                                                                   p, beta, partials);
-                return cudaGetLastError();
-            }
+template <int N>
+struct Bp35PcgF32Launch {
+    static cudaError_t run(int64_t E, const float *G, double lambda, const float *z, float *p, const double *beta,
+                           float *Ap, double *partials, cudaStream_t s, double *status) {
+        if constexpr (bp35_streamed<N, true, float>()) {
+            return launch_stream35<N, true>(E, G, lambda, nullptr, Ap, z, p, beta, partials, s, nullptr, status);
+        } else if constexpr (bp35_streamed1<N, true, float>()) {
+            return launch_stream35_1<N, true>(E, G, lambda, nullptr, Ap, z, p, beta, partials, s, nullptr, status);
+        } else {
+            using C = Bp35Cfg<float, N>;
+            const int64_t blocks = (E + C::EPB - 1) / C::EPB;
+            bp35_fn<float, N, true>()<<<(unsigned)blocks, C::threads, C::smem, s>>>(E, G, lambda, nullptr, Ap, z, p,
+                                                                                   beta, partials);
+            return cudaGetLastError();
         }
-    };
+    }
 };
 
 template <int N>
 struct Bp35Blocks {
-    static cudaError_t run(int64_t E, int which, int64_t *out) {
-        using C = Bp35Cfg<double, N>;
+    static cudaError_t run(int64_t E, int64_t *out) {
         using F = Bp35Cfg<float, N>;
-        const int64_t a = (E + C::EPB - 1) / C::EPB;
         int64_t b = (E + F::EPB - 1) / F::EPB;
         if constexpr (bp35_streamed<N, true, float>()) {
             using S = Bp35Stream<N, true>;
@@ -130,7 +103,7 @@ struct Bp35Blocks {
         } else if constexpr (bp35_streamed1<N, true, float>()) {
             b = stream_grid35(E, Bp35Stream1<N, true, float>::blocks_per_sm);
         }
-        *out = which == 0 ? a : which == 1 ? b : (a > b ? a : b);
+        *out = b;
         return cudaSuccess;
     }
 };
@@ -143,9 +116,7 @@ struct Bp35Prepare {
                                     Bp35Cfg<T, N>::smem);
     }
     static cudaError_t run() {
-        cudaError_t e = one<double, false>();
-        if (e == cudaSuccess) e = one<double, true>();
-        if (e == cudaSuccess) e = one<float, false>();
+        cudaError_t e = one<float, false>();
         if (e == cudaSuccess) e = one<float, true>();
         // the stream kernels keep all operands in shared memory: they ask
         // for the largest carveout
@@ -162,44 +133,29 @@ FEM_DEFINE_FOLD_UPLOAD(upload_fold_bp35_tu)
 
 FEM_DEFINE_WAIT_COUNTER(wait_timeouts_bp35)
 
-cudaError_t launch_bp35(const fem_basis *b, int64_t E, const double *G, double lambda, const double *q,
-                        double *Aq, cudaStream_t s) {
-    return dispatch_degree<Bp35Launch>(b->host.N, E, G, lambda, q, Aq, s);
-}
-
 cudaError_t launch_bp35_f32(const fem_basis *b, int64_t E, const float *G, double lambda, const float *q,
                             float *Aq, cudaStream_t s) {
     return dispatch_degree<Bp35F32Launch>(b->host.N, E, G, lambda, q, Aq, s);
 }
 
-cudaError_t launch_bp35_pcg(const fem_basis *b, int64_t E, const double *G, double lambda, const double *z,
-                            double *p, const double *beta, double *Ap, double *partials, cudaStream_t s) {
-    return dispatch_degree<Bp35PcgLaunchT<double>::L>(b->host.N, E, G, lambda, z, p, beta, Ap, partials, s,
-                                                       (double *)nullptr);
-}
-
 cudaError_t launch_bp35_pcg_f32(const fem_basis *b, int64_t E, const float *G, double lambda, const float *z,
                                 float *p, const double *beta, float *Ap, double *partials, cudaStream_t s,
                                 double *status) {
-    return dispatch_degree<Bp35PcgLaunchT<float>::L>(b->host.N, E, G, lambda, z, p, beta, Ap, partials, s, status);
-}
-
-int64_t bp35_max_blocks(int N, int64_t E) {
-    int64_t out = 0;
-    dispatch_degree<Bp35Blocks>(N, E, 2, &out);
-    return out;
+    return dispatch_degree<Bp35PcgF32Launch>(b->host.N, E, G, lambda, z, p, beta, Ap, partials, s, status);
 }
 
 int64_t bp35_blocks(int N, int64_t E, bool f32) {
+    if (!f32) return bp35_fx_blocks(N, E);
     int64_t out = 0;
-    dispatch_degree<Bp35Blocks>(N, E, f32 ? 1 : 0, &out);
+    dispatch_degree<Bp35Blocks>(N, E, &out);
     return out;
 }
 
 cudaError_t prepare_bp35(int N, const double *fold_table) {
     cudaError_t e = upload_fold_bp35_tu(fold_table);
     if (e != cudaSuccess) return e;
-    return dispatch_degree<Bp35Prepare>(N);
+    e = dispatch_degree<Bp35Prepare>(N);
+    return e == cudaSuccess ? prepare_bp35_fx(N, fold_table) : e;
 }
 
 namespace {

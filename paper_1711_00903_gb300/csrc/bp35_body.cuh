@@ -1,6 +1,5 @@
-// Body of the BP3.5 kernels as a device function, shared by the stand-alone
-// kernels (bp35.cu) and the batched persistent kernel (batch.cu).  See
-// bp35.cu for the algorithm and the GB300 design.
+// Body of the FP32 BP3.5 kernels (FP32 and FP16 factors) as a device function.
+// See bp35.cu for the algorithm and the GB300 design.
 #pragma once
 
 #include <type_traits>
@@ -58,14 +57,13 @@ struct Bp35Layout {
     static constexpr int oD = fold_offset(N, kFoldD), oDT = fold_offset(N, kFoldDT);
 };
 
-// Elements per block of the stand-alone kernels: as many as fit 256 threads
-// under the shared-memory budget (512 for FP64 from N = 8 on, measured 9 %
-// faster at N = 9 and 11; 128 for FP32 at N = 10, 6 % faster).
+// Elements per block of the block kernels: as many as fit 256 threads under
+// the shared-memory budget (128 at N = 10, 6 % faster).
 template <typename T, int N>
 struct Bp35Cfg
     : Bp35Layout<T, N,
                  pick_epb(N + 1, 3 * Box<N + 1, N + 1, N + 1>::size * (int)sizeof(T),
-                          sizeof(T) == 8 ? (N >= 8 ? 512 : 256) : (N == 10 ? 128 : 256))> {
+                          N == 10 ? 128 : 256)> {
 };
 
 // The operator on elements [e0, e0 + nel) (nel <= EPB) whose input field is
@@ -219,7 +217,6 @@ __device__ __forceinline__ void bp35_block(unsigned char *smem_raw, int64_t e0, 
 // from the operator sweep on GB300.
 template <typename T, int N>
 constexpr int bp35_min_blocks() {
-    if (sizeof(T) == 8) return N >= 10 ? 3 : 0;
     return N == 15 ? 3 : 0;
 }
 

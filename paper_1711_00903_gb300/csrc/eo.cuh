@@ -41,7 +41,16 @@ namespace fem {
 // One constant table per translation unit and precision (no relocatable
 // device code); every TU that uses them uploads the same contents at basis
 // setup.
+//
+// Translation units whose constant bank holds the fixed-point tables of
+// fx.cuh (FEM_FX_TABLES) keep this FP64 table in global memory: their FP64
+// lines are the exception there, and a load per FMA hides behind the FP64
+// pipe (2 per clock per SM).
+#ifdef FEM_FX_TABLES
+static __device__ double c_fold[kFoldTotal];
+#else
 static __constant__ double c_fold[kFoldTotal];
+#endif
 static __constant__ float2 c_fold32p[kFoldPairTotal];
 
 // FP32 form of eo_apply below (the pair table, OFF its folded offset).

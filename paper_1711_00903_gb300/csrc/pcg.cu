@@ -499,7 +499,6 @@ cudaError_t launch_bp35_pcg(const fem_basis *b, int64_t E, const double *G, doub
 cudaError_t launch_bp35_pcg_f32(const fem_basis *b, int64_t E, const float *G, double lambda, const float *z,
                                 float *p, const double *beta, float *Ap, double *partials, cudaStream_t s,
                                 double *status);
-int64_t bp35_max_blocks(int N, int64_t E);
 int64_t bp35_blocks(int N, int64_t E, bool f32);
 cudaError_t launch_bp35(const fem_basis *b, int64_t E, const double *G, double lambda, const double *q, double *Aq,
                         cudaStream_t s);

@@ -1,0 +1,149 @@
+"""The FP64 operators on the integer pipe (csrc/fx.cuh) where their rules
+change hands: element scales from 2^-900 to 2^900, elements that hold values
+of many magnitudes, zeros, spikes, NaN and Inf (which go through FP64 lines),
+flat and indefinite factors, every degree, element counts around the block
+sizes.  Against the oracle, node by node.
+
+Bar: |y - y_oracle| <= 8 (1.5 n + 17) 2^-53 b, with b the same operator on
+absolute values and on operators folded even-odd as FP64 lines evaluate them,
+(|A[a][i]| + |A[a][Q-1-i]|) for A[a][i]: an FP64 evaluation makes at most
+about n/2 + 3 roundings per contraction on the longest chain (three
+contractions in BP3.5), 8 in the chain rule and the sums, for each side,
+times 4 for what the two evaluations order differently."""
+import numpy as np
+import pytest
+
+import fem_synth
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _fem():
+    import paper_1711_00903_gb300 as fem
+    return fem
+
+
+def _dev(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).to("cuda")
+
+
+def _along(A, u, axis):
+    return np.moveaxis(np.tensordot(A, u, axes=(1, axis)), 0, axis)
+
+
+def _folded_abs(A):
+    return np.abs(A) + np.abs(A[:, ::-1])
+
+
+def _stiff_abs(D, G, u):
+    k = u.shape[-1]
+    g = np.abs(G).reshape(-1, 7, k, k, k)
+    D, DT = _folded_abs(D), _folded_abs(D.T)
+    ur, us, ut = _along(D, u, 3), _along(D, u, 2), _along(D, u, 1)
+    wr = g[:, 0] * ur + g[:, 1] * us + g[:, 2] * ut
+    ws = g[:, 1] * ur + g[:, 3] * us + g[:, 4] * ut
+    wt = g[:, 2] * ur + g[:, 4] * us + g[:, 5] * ut
+    return _along(DT, wr, 3) + _along(DT, ws, 2) + _along(DT, wt, 1), g[:, 6]
+
+
+class Op:
+    """BP3.5 with its factors, oracle and bound."""
+
+    chain = 1.5
+
+    def __init__(self, N):
+        self.N, self.n, self.b = N, N + 1, oracle.Basis(N)
+
+    def factors(self, verts):
+        return oracle.geofacs(self.N, 2, verts)[0]
+
+    def oracle(self, geo, q):
+        return oracle.bp35(self.N, geo, 0.37, q)
+
+    def apply(self, geo, q):
+        fem = _fem()
+        return fem.fem_bp35_apply(fem.fem_basis_setup(self.N), _dev(geo), 0.37, _dev(q)).cpu().numpy()
+
+    def bound(self, geo, q):
+        u = np.abs(q).reshape(-1, self.n, self.n, self.n)
+        s, wj = _stiff_abs(self.b.D, geo, u)
+        return (s + 0.37 * wj * u).reshape(q.shape)
+
+    @property
+    def tol(self):
+        return 8 * (self.chain * self.n + 17) * 2.0 ** -53
+
+
+OPS = {"bp35": Op}
+
+
+def _check(op, geo, q):
+    got, ref = op.apply(geo, q), op.oracle(geo, q)
+    np.testing.assert_array_equal(np.isfinite(got), np.isfinite(ref))
+    fine = np.isfinite(ref)
+    with np.errstate(invalid="ignore", over="ignore"):
+        assert np.all(np.abs(got - ref)[fine] <= (op.tol * op.bound(geo, q))[fine])
+    return got
+
+
+def _elements(op, seed=5):
+    """Eleven elements: ordinary ones and each kind that changes the path."""
+    rng = np.random.default_rng(seed)
+    verts = fem_synth.box_mesh(3, 2, 2, seed=seed)[:11].copy()
+    geo = op.factors(verts)
+    NP = op.n ** 3
+    q = rng.uniform(-1, 1, (11, NP))
+    i = np.arange(NP)
+    q[1] = 0.0
+    q[2, rng.integers(NP)] = 1e12                                       # one value far above the rest
+    q[3] *= 10.0 ** -(2.0 * (i % op.n + (i // op.n) % op.n + i // op.n ** 2))  # decay in every direction
+    q[4] = 0.0
+    q[4, rng.integers(NP)] = 1.0                                        # a unit vector
+    q[5, rng.integers(NP)] = np.nan
+    q[6, rng.integers(NP)] = np.inf
+    q[7] *= 2.0 ** 900
+    q[8] *= 2.0 ** -900
+    geo[9] = -geo[9]                                                    # not positive definite
+    q[10].reshape(op.n, op.n, op.n)[0, 0, :] = 1e-17                    # an edge of near-zeros
+    return geo, q
+
+
+@pytest.mark.parametrize("name", sorted(OPS))
+@pytest.mark.parametrize("N", range(1, 16))
+def test_elements_of_every_kind(name, N):
+    op = OPS[name](N)
+    geo, q = _elements(op)
+    got = _check(op, geo, q)
+    # an element's result does not depend on its neighbours in the block
+    for e in (0, 3, 10):
+        np.testing.assert_array_equal(op.apply(geo[e:e + 1], q[e:e + 1])[0], got[e])
+
+
+@pytest.mark.parametrize("name", sorted(OPS))
+@pytest.mark.parametrize("N", [1, 4, 7, 10, 15])
+def test_flat_and_scaled_elements(name, N):
+    op = OPS[name](N)
+    rng = np.random.default_rng(N)
+    verts = fem_synth.box_mesh(3, 1, 1, seed=N)
+    q = rng.uniform(-1, 1, (3, op.n ** 3))
+    for scale in ((1, 1, 1e-4), (1e3, 1, 1), (1e-3, 1e-3, 1e-3)):
+        _check(op, op.factors(np.ascontiguousarray(verts * np.array(scale))), q)
+    geo = op.factors(verts)
+    got = op.apply(geo, q)
+    for k in (-200, 40, 200):  # a power of two scales the result exactly
+        np.testing.assert_array_equal(op.apply(geo, np.ldexp(q, k)), np.ldexp(got, k))
+        np.testing.assert_array_equal(op.apply(np.ldexp(geo, k), q), np.ldexp(got, k))
+
+
+@pytest.mark.parametrize("name", sorted(OPS))
+@pytest.mark.parametrize("N", [1, 2, 3, 5, 6, 8, 9, 12])
+def test_element_counts_around_the_blocks(name, N):
+    op = OPS[name](N)
+    verts = fem_synth.box_mesh(5, 5, 3, seed=N)
+    geo = op.factors(verts)
+    q = np.random.default_rng(N).uniform(-1, 1, (75, op.n ** 3))
+    full = _check(op, geo, q)
+    for E in (1, 2, 3, 7, 31, 32, 33):
+        np.testing.assert_array_equal(op.apply(geo[:E], q[:E]), full[:E])
