@@ -5,8 +5,8 @@
 // one mesh (EPB chosen per degree for the launch's block size).  A grid of
 // (resident blocks per SM x SMs) persistent blocks pulls groups of tasks
 // from a global counter (one atomicAdd per group) and runs each task with
-// the same device functions as the stand-alone kernels (bp35_body.cuh,
-// bp30_body.cuh), so every element's result is bit-identical to the
+// the same device functions as the stand-alone kernels (bp35_fx.cuh,
+// bp30_fx.cuh), so every element's result is bit-identical to the
 // per-mesh calls.  Tasks are ordered by decreasing cost per element by
 // default, so that the expensive high-degree work starts first and the tail
 // is made of cheap tasks.
@@ -23,7 +23,7 @@
 #include <new>
 #include <vector>
 
-#include "bp30_body.cuh"
+#include "bp30_fx.cuh"
 #include "bp30_point.cuh"
 #include "bp35_fx.cuh"
 #include "bp35_point.cuh"
@@ -63,7 +63,7 @@ struct Epb35 {
 template <int THREADS, int N>
 struct Epb30 {
     static constexpr int m = N + 2;
-    static constexpr int per = 3 * Box<m, m, m>::size * 8;
+    static constexpr int per = 4 * Box<m, m, m>::size * 8;
     static constexpr int a = THREADS / (m * m), b = kBatchSmemBudget / per;
     static constexpr int v = (a < b ? a : b) > 0 ? (a < b ? a : b) : 1;
 };
@@ -71,7 +71,7 @@ struct Epb30 {
 template <int THREADS, int N>
 constexpr int batch_smem_n() {
     constexpr int s35 = Fx35Layout<N, Epb35<THREADS, N>::v>::smem;
-    constexpr int s30 = Bp30Layout<N, Epb30<THREADS, N>::v>::smem;
+    constexpr int s30 = Fx30Layout<N, Epb30<THREADS, N>::v>::smem;
     constexpr int sp = N <= kBatchMaxPointN ? Bp30Point<N>::smem : 0;
     constexpr int sp35 = N <= kBatchMaxPointN35 ? Bp35Point<N>::smem : 0;
     constexpr int s = s35 > s30 ? s35 : s30;
@@ -115,7 +115,8 @@ __device__ __noinline__ void task35(unsigned char *smem, const BatchTask tk, con
 }
 template <int THREADS, int K>
 __device__ __noinline__ void task30(unsigned char *smem, const BatchTask tk, const BatchMesh M) {
-    bp30_block<K, Epb30<THREADS, K>::v>(reinterpret_cast<double *>(smem), tk.e0, tk.nel, M.G, M.lambda, M.q, M.out);
+    bp30_fx_block<K, Epb30<THREADS, K>::v, false, false>(smem, tk.e0, tk.nel, M.G, M.lambda, M.q, M.out, nullptr, nullptr,
+                                                         nullptr, nullptr, nullptr);
 }
 // the same tasks in the point layouts: their elements one after the other
 template <int THREADS, int K>
@@ -134,7 +135,11 @@ __device__ __noinline__ void task35_point(unsigned char *smem, const BatchTask t
 }
 
 template <int THREADS>
-__global__ void __launch_bounds__(THREADS)
+// Two resident blocks per SM (a register cap of 128 at 256 threads, 64 at
+// 512): 24 meshes of degree 2..10 measured 1574 us with the compiler's own
+// choice at 256 threads, 1048 with two blocks and 1145 with three; 1580, 1376
+// and 1950 at 512.
+__global__ void __launch_bounds__(THREADS, 2)
 batch_kernel(const BatchMesh *__restrict__ meshes, const BatchTask *__restrict__ tasks, int ntasks, int group,
              int layout, int *__restrict__ counter) {
     extern __shared__ __align__(16) unsigned char smem[];

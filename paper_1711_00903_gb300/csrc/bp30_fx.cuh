@@ -1,0 +1,673 @@
+// BP1.0, BP3.0 and both in one pass in FP64 with their arithmetic on the
+// integer multiply-add pipe (fx.cuh), shared by the stand-alone kernels
+// (bp1_fx.cu, bp30_fx.cu) and the batched persistent kernel (batch.cu).
+//
+// The scales follow the element's data as in bp35_fx.cuh:
+//   1. q, scaled by the element's largest |q| to 59 or 60 bits, through the
+//      three interpolations (each output is a mix of the whole element, so
+//      one scale serves it), scaled up once more before the third;
+//   2. BP1.0: times wJ (62 bits, without its weights' powers of two), through
+//      the three projections, which carry the weights: the second takes its
+//      input scaled up by the element's largest value, the third by the
+//      line's (three in a row at the worst case's scale would lose 6 to 9
+//      bits);
+//   3. BP3.0: derivatives, scaled up by their largest value; chain rule with
+//      the factors scaled to 62 bits; transposes, each line scaled up by its
+//      largest value; their sum with lambda wJ q, aligned, scaled up by its
+//      largest value; the three projections.
+// BP1.0 computed beside BP3.0 takes the same steps on the same numbers as
+// alone, and BP3.0 the same with and without it: equal bits.
+//
+// An element goes through FP64 instead (bp1_element64, bp30_element64) when
+// its values are not finite or extreme, when one of its eight octants holds
+// no value near its largest (the FP64 result there would keep digits that
+// the element's scale cuts off), when a point's factors are far below the
+// element's largest, or when the factors are not positive definite; element
+// by element, so a result does not depend on the block's other elements.
+//
+// What bounds it: integer multiply-adds and, between barriers, latency; see
+// bp30_fx.cu and bp1_fx.cu for the measured rates.
+#pragma once
+
+#include "bp30_body.cuh"  // Bp30Layout
+#include "fx.cuh"
+#include "fx_point.cuh"
+
+namespace fem {
+namespace {
+
+// How far (in bits) below the element's largest value an octant's largest
+// may lie.  At N = 1, where an octant is one node (of a field that vanishes
+// on a face, a zero), every node's result holds at least an eighth of every
+// other's: any range will do.
+__host__ __device__ constexpr int fx30_octant_range(int N) { return N == 1 ? 2047 : kFxRange; }
+
+// Slots of an element's statistics: the eight octants of q, the largest wJ,
+// Grr, Gss, Gtt, derivative and sum at the Gauss points, whether the element
+// is left to FP64 (BP1.0, BP3.0), the largest value after the projection along
+// t (BP1.0, BP3.0) and after the interpolation along s, and the largest scale
+// of a transposed line (as 63 - its scale-up).
+enum { kFxW = 8, kFxG = 9, kFxU = 12, kFxX = 13, kFxLeft1 = 14, kFxLeft30 = 15, kFxT1 = 16, kFxT30 = 17, kFxI = 18, kFxH = 19, kFx30Stats = 20 };
+
+// A line of Q values at from(l), contracted, its outputs to put(l, y).
+template <int P, int Q, int SIG, int OFF, class L, class F>
+__device__ __forceinline__ void fx_line(L &&from, F &&put) {
+    long long x[Q];
+#pragma unroll
+    for (int l = 0; l < Q; l++) x[l] = from(l);
+    fx_apply<P, Q, SIG, OFF>(x, put);
+}
+
+// g x / 2^62 of a factor below 2^62 (halves) and |x| < 2^60.
+__device__ __forceinline__ long long fx_mul(int gh, int gl, long long x) {
+    const int xh = fx_hi(x), xl = fx_lo(x);
+    return (mul_wide(gh, xh) << 2) + (mad_wide(gl, xh, mad_wide(gh, xl, 1ll << 29)) >> 30);
+}
+
+// Scale-up of the values before the interpolation along t.
+template <int N>
+__device__ __forceinline__ int fx30_up(const unsigned *st) {
+    return max(0, fx_qbits30(N) - 32 - fx_top((int)st[kFxI]));
+}
+
+// The high word's largest magnitude over the values seen.
+struct FxMost {
+    int hi = 0, lo = 0;
+    __device__ __forceinline__ void see(long long x) {
+        hi = max(hi, (int)(x >> 32));
+        lo = min(lo, (int)(x >> 32));
+    }
+    __device__ __forceinline__ int value() const { return max(hi, ~lo); }
+};
+
+// The projections of EPB elements along s (box X of t-projected values, whose
+// largest is at `slot` of the statistics, to box Y) and along r (box Y to the
+// output, exponent(e) that of the s-projected values without their scale-up),
+// for elements not left to FP64.
+template <int N, int EPB_, class B1, class B2>
+__device__ __forceinline__ void fx30_project_s(int nel, const long long *X, long long *Y, int per, const unsigned *stats,
+                                               int slot) {
+    constexpr int n = N + 1, m = N + 2;
+    for_tasks<m * n, EPB_>(nel, [&](int e, int t) {
+        const long long *Xe = X + e * per;
+        long long *Ye = Y + e * per;
+        const int i = t % m, k = t / m, up = max(0, kFxBits30 - 32 - fx_top((int)stats[e * kFx30Stats + slot]));
+        fx_line<n, m, 1, fold_offset(N, kFoldIT)>([&](int l) { return Xe[B2::at(i, l, k)] << up; },
+                                                  [&](int l, long long y) { Ye[B1::at(i, l, k)] = y; });
+    });
+}
+template <int N, int EPB_, class B1, class F, class O>
+__device__ __forceinline__ void fx30_project_r(int nel, const long long *Y, int per, const unsigned *stats, int slot,
+                                               int left, F &&exponent, O &&out) {
+    constexpr int n = N + 1, m = N + 2;
+    for_tasks<n * n, EPB_>(nel, [&](int e, int t) {
+        const unsigned *se = stats + e * kFx30Stats;
+        if (se[left] != 0) return;
+        const long long *Ye = Y + e * per;
+        const int j = t % n, k = t / n;
+        long long x[m];
+#pragma unroll
+        for (int l = 0; l < m; l++) x[l] = Ye[B1::at(l, j, k)];
+        const int h = max(0, kFxBits30 - 32 - fx_top(fx_line_max(x)));
+#pragma unroll
+        for (int l = 0; l < m; l++) x[l] <<= h;
+        const int k2 = exponent(e) - max(0, kFxBits30 - 32 - fx_top((int)se[slot])) - h + c_fxd[N].wn[j] + c_fxd[N].wn[k];
+        fx_apply<n, m, 1, fold_offset(N, kFoldIT)>(
+            x, [&](int l, long long y) { out(e, t, l, fx_to_double(y, k2 + c_fxd[N].wn[l])); });
+    });
+}
+
+// Loads the field of column (i, j) = r of an element (r < n^2; PCG: p <- z +
+// beta p, stored) and folds its largest values into the octants' slots; a
+// middle node belongs to both halves.
+template <int N, bool PCG>
+__device__ __forceinline__ void fx30_load(double (&qv)[N + 1], int64_t g0, int r, const double *__restrict__ q,
+                                          const double *__restrict__ z, double *p, const double *__restrict__ beta,
+                                          unsigned *st) {
+    constexpr int n = N + 1, nn = n * n;
+    if (PCG) {
+        const double bt = *beta;
+#pragma unroll
+        for (int k = 0; k < n; k++) {
+            const int64_t g = g0 + k * nn;
+            qv[k] = (bt == 0.0) ? z[g] : fma(bt, p[g], z[g]);
+            p[g] = qv[k];
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < n; k++) qv[k] = __ldg(q + g0 + k * nn);
+    }
+    unsigned lo = 0, hi = 0;
+#pragma unroll
+    for (int k = 0; k < n; k++) {
+        const unsigned a = (unsigned)fx_abs_hi(qv[k]);
+        if (k <= N / 2) lo = max(lo, a);
+        if (k >= n / 2) hi = max(hi, a);
+    }
+    const int i = r % n, j = r / n;
+#pragma unroll
+    for (int o = 0; o < 4; o++) {
+        const bool in_i = (o & 1) ? i >= n / 2 : i <= N / 2, in_j = (o & 2) ? j >= n / 2 : j <= N / 2;
+        if (in_i && in_j) {
+            atomicMax(st + o, lo);
+            atomicMax(st + 4 + o, hi);
+        }
+    }
+}
+
+// The element's scale from its octants: |q| < 2^kq; left: the element is not
+// held to one scale.
+template <int N>
+__device__ __forceinline__ int fx30_scale(const unsigned *st, bool *left) {
+    unsigned most = 0, least = 0x7fffffffu;
+#pragma unroll
+    for (int o = 0; o < 8; o++) {
+        most = max(most, st[o]);
+        least = min(least, st[o]);
+    }
+    const int e = (int)(most >> 20);
+    *left = most != 0 && (e < 64 || e == 0x7ff || (int)(least >> 20) < e - fx30_octant_range(N));
+    return most ? e - 1022 : 0;
+}
+
+// Largest exponents (high words without the weights) of `planes` factor
+// planes at column r of the Gauss points (weights of the column wab).
+template <int N, int planes>
+__device__ __forceinline__ void fx30_scan(const double *Ge, const int (&plane)[planes], int wab, unsigned *slots) {
+    constexpr int m = N + 2, mm = m * m, MP = m * mm;
+    const int *Gi = reinterpret_cast<const int *>(Ge) + 1;  // high words
+    int most[planes];
+#pragma unroll
+    for (int h = 0; h < planes; h++) most[h] = 0;
+#pragma unroll 4
+    for (int c = 0; c < m; c++) {
+        const int w = c_fxd[N].wm[c] << 20;
+#pragma unroll
+        for (int h = 0; h < planes; h++) most[h] = max(most[h], __ldg(Gi + 2 * (plane[h] * MP + c * mm)) - w);
+    }
+#pragma unroll
+    for (int h = 0; h < planes; h++) fx_element_max<mm>(slots + h, (unsigned)(most[h] - (wab << 20)));
+}
+
+// BP1.0's step at a Gauss point: wJ qg, with wJ scaled by 2^(62 - kw).
+// bw: kw + 1022 plus the point's weight exponents.  A wJ that is not positive
+// or far below the element's largest raises far, a larger or non-finite one
+// lowers least.
+__device__ __forceinline__ long long fx30_mass(double wj, int bw, long long qg, int &far, int &least) {
+    const int s = bw - (__double2hiint(wj) >> 20);
+    far = max(far, s);
+    least = min(least, s);
+    int gh, gl;
+    fx_diagonal(wj, s, gh, gl);
+    return fx_mul(gh, gl, qg);
+}
+
+// Exponent of BP1.0's projected values (without the scale-ups) from an
+// element's statistics.
+template <int N>
+__device__ __forceinline__ int fx1_exponent(const unsigned *st) {
+    bool left;
+    return fx30_scale<N>(st, &left) - fx_qbits30(N) - fx30_up<N>(st) + 3 * (c_fxd[N].tau[kFoldI] + c_fxd[N].tau[kFoldIT]) +
+           (int)(st[kFxW] >> 20) - 1022;
+}
+
+// Algorithm 3 in FP64 on one element by the whole block, sizes at run time
+// (fx_line64); smem: at least 2 m^3 doubles (rows of m, or m + 1 for even m).
+__device__ __noinline__ void bp1_element64(double *smem, int n, int oI, int oIT, const double *wJ, const double *q,
+                                           double *Mq) {
+    const int m = n + 1, mm = m * m, nn = n * n, NP = nn * n, sj = m | 1, sk = sj * m;
+    double *X = smem, *Y = smem + sk * m;
+    __syncthreads();  // the shared memory is free
+    for (int t = threadIdx.x; t < NP; t += blockDim.x) X[t % n + sj * ((t / n) % n) + sk * (t / nn)] = q[t];
+    __syncthreads();
+    for (int t = threadIdx.x; t < nn; t += blockDim.x) {
+        const int o = sj * (t % n) + sk * (t / n);
+        fx_line64(X + o, 1, Y + o, 1, m, n, 1, oI);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < m * n; t += blockDim.x) {
+        const int o = t % m + sk * (t / m);
+        fx_line64(Y + o, sj, X + o, sj, m, n, 1, oI);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < mm; t += blockDim.x) {
+        const int o = t % m + sj * (t / m);
+        double g[kMaxQ];
+        fx_line64(X + o, sk, g, 1, m, n, 1, oI);
+        for (int c = 0; c < m; c++) g[c] *= wJ[t + c * mm];
+        fx_line64(g, 1, X + o, sk, n, m, 1, oIT);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < m * n; t += blockDim.x) {
+        const int o = t % m + sk * (t / m);
+        fx_line64(X + o, sj, Y + o, sj, n, m, 1, oIT);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < nn; t += blockDim.x)
+        fx_line64(Y + sj * (t % n) + sk * (t / n), 1, Mq + t * n, 1, n, m, 1, oIT);
+}
+
+// Algorithm 5 in FP64 on one element by the whole block (at least m^2
+// threads); smem: at least 3 m^3 doubles as above.
+__device__ __noinline__ void bp30_element64(double *smem, int n, int oI, int oIT, int oDt, int oDtT, const double *G,
+                                            double lambda, const double *q, double *Aq) {
+    const int m = n + 1, mm = m * m, MP = mm * m, nn = n * n, NP = nn * n, sj = m | 1, sk = sj * m, size = sk * m;
+    double *A = smem, *B = A + size, *C = B + size;
+    __syncthreads();  // the shared memory is free
+    for (int t = threadIdx.x; t < NP; t += blockDim.x) B[t % n + sj * ((t / n) % n) + sk * (t / nn)] = q[t];
+    __syncthreads();
+    for (int t = threadIdx.x; t < nn; t += blockDim.x) {
+        const int o = sj * (t % n) + sk * (t / n);
+        fx_line64(B + o, 1, C + o, 1, m, n, 1, oI);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < m * n; t += blockDim.x) {
+        const int o = t % m + sk * (t / m);
+        fx_line64(C + o, sj, B + o, sj, m, n, 1, oI);
+    }
+    __syncthreads();
+    const int r = threadIdx.x, u = r % m, v = r / m, oc = u + sj * v, orr = sj * u + sk * v, os = u + sk * v;
+    if (r < mm) fx_line64(B + oc, sk, A + oc, sk, m, n, 1, oI);
+    __syncthreads();
+    double ut[kMaxQ], acc[kMaxQ];
+    if (r < mm) {
+        fx_line64(A + orr, 1, B + orr, 1, m, m, -1, oDt);
+        fx_line64(A + os, sj, C + os, sj, m, m, -1, oDt);
+        fx_line64(A + oc, sk, ut, 1, m, m, -1, oDt);
+    }
+    __syncthreads();
+    if (r < mm) {
+        for (int c = 0; c < m; c++) {
+            const int s = oc + sk * c;
+            const double *g = G + r + c * mm, qr = B[s], qs = C[s], qt = ut[c];
+            B[s] = g[0] * qr + g[MP] * qs + g[2 * MP] * qt;
+            C[s] = g[MP] * qr + g[3 * MP] * qs + g[4 * MP] * qt;
+            ut[c] = g[2 * MP] * qr + g[4 * MP] * qs + g[5 * MP] * qt;
+        }
+        fx_line64(ut, 1, acc, 1, m, m, -1, oDtT);
+        if (lambda != 0.0)
+            for (int c = 0; c < m; c++) acc[c] = fma(lambda * G[6 * MP + r + c * mm], A[oc + sk * c], acc[c]);
+    }
+    __syncthreads();
+    if (r < mm) {
+        fx_line64(B + orr, 1, B + orr, 1, m, m, -1, oDtT);
+        fx_line64(C + os, sj, C + os, sj, m, m, -1, oDtT);
+    }
+    __syncthreads();
+    if (r < mm) {
+        for (int c = 0; c < m; c++) acc[c] += B[oc + sk * c] + C[oc + sk * c];
+        fx_line64(acc, 1, A + oc, sk, n, m, 1, oIT);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < m * n; t += blockDim.x) {
+        const int o = t % m + sk * (t / m);
+        fx_line64(A + o, sj, B + o, sj, n, m, 1, oIT);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < nn; t += blockDim.x)
+        fx_line64(B + sj * (t % n) + sk * (t / n), 1, Aq + t * n, 1, n, m, 1, oIT);
+}
+
+// ---------------------------------------------------------------- BP1.0
+
+// Shared memory of EPB elements: a box for q, the twice interpolated and the
+// once projected field, one for the once interpolated and the twice
+// projected, and the statistics.  (bp1_element64 needs two m^3 boxes.)
+template <int N, int EPB_>
+struct Fx1Layout {
+    static constexpr int n = N + 1, m = N + 2, nn = n * n, mm = m * m, NP = nn * n, MP = mm * m, EPB = EPB_;
+    using B0 = Box<n, n, n>;
+    using B1 = Box<m, n, n>;
+    using B2 = Box<m, m, n>;
+    static constexpr int SA = B0::size > B2::size ? B0::size : B2::size, per = SA + B1::size;
+    static constexpr int threads = ((mm * EPB + 31) / 32) * 32;
+    // the statistics lie past the boxes of either path
+    static constexpr int boxes = EPB * per * 8, boxes64 = 2 * Box<m, m, m>::size * 8;
+    static constexpr int off_stats = boxes > boxes64 ? boxes : boxes64;
+    static constexpr int smem = off_stats + EPB * kFx30Stats * 4;
+};
+
+// BP1.0 of elements [e0, e0 + nel) by the whole block (blockDim.x >=
+// Layout::threads); wJ: m^3 values per element.
+template <int N, int EPB_>
+__device__ __forceinline__ void bp1_fx_block(unsigned char *smem_raw, int64_t e0, int nel, const double *__restrict__ wJ,
+                                             const double *__restrict__ q, double *__restrict__ Mq) {
+    using C = Fx1Layout<N, EPB_>;
+    using B0 = typename C::B0;
+    using B1 = typename C::B1;
+    using B2 = typename C::B2;
+    constexpr int n = C::n, m = C::m, nn = C::nn, mm = C::mm, NP = C::NP, MP = C::MP, K = kFx30Stats, QB = fx_qbits30(N);
+    constexpr int oI = fold_offset(N, kFoldI), oIT = fold_offset(N, kFoldIT);
+    const int el = threadIdx.x / mm, r = threadIdx.x - el * mm;
+    const bool act = el < nel;
+    const int a = r % m, b = r / m;
+    long long *boxes = reinterpret_cast<long long *>(smem_raw);
+    unsigned *stats = reinterpret_cast<unsigned *>(smem_raw + C::off_stats), *st = stats + el * K;
+    if (threadIdx.x == 0) prefetch_l2(wJ + e0 * MP, (long long)nel * MP * 8);
+    for (int t = threadIdx.x; t < EPB_ * K; t += blockDim.x) stats[t] = 0;
+    __syncthreads();
+
+    double qv[n];
+    const bool col = act && r < nn;
+    if (col) fx30_load<N, false>(qv, (e0 + el) * NP + r, r, q, nullptr, nullptr, nullptr, st);
+    __syncthreads();
+    int kq = 0;
+    if (act) {
+        bool left;
+        kq = fx30_scale<N>(st, &left);
+        if (col) {
+#pragma unroll
+            for (int k = 0; k < n; k++) {
+                const int e = (__double2hiint(qv[k]) >> 20) & 0x7ff;
+                left = left || (kq == 0 && e == 0 && (fx_abs_hi(qv[k]) | __double2loint(qv[k])) != 0);
+                boxes[el * C::per + B0::at(r % n, r / n, k)] = fx_from_double<QB>(qv[k], kq + 1022 - e);
+            }
+        }
+        if (left) st[kFxLeft1] = 1;
+    }
+    __syncthreads();
+
+    // interpolation along r and s
+    for_tasks<nn, EPB_>(nel, [&](int e, int t) {
+        const long long *X = boxes + e * C::per;
+        long long *Y = boxes + e * C::per + C::SA;
+        const int j = t % n, k = t / n;
+        fx_line<m, n, 1, oI>([&](int l) { return X[B0::at(l, j, k)]; }, [&](int l, long long y) { Y[B1::at(l, j, k)] = y; });
+    });
+    const int wab = act ? c_fxd[N].wm[a] + c_fxd[N].wm[b] : 0;
+    if (act) fx30_scan<N, 1>(wJ + (e0 + el) * MP + r, {0}, wab, st + kFxW);
+    __syncthreads();
+    for_tasks<m * n, EPB_>(nel, [&](int e, int t) {
+        const long long *Y = boxes + e * C::per + C::SA;
+        long long *X = boxes + e * C::per;
+        const int i = t % m, k = t / m;
+        FxMost most;
+        fx_line<m, n, 1, oI>([&](int l) { return Y[B1::at(i, l, k)]; },
+                             [&](int l, long long y) {
+                                 X[B2::at(i, l, k)] = y;
+                                 most.see(y);
+                             });
+        atomicMax(stats + e * K + kFxI, (unsigned)most.value());
+    });
+    __syncthreads();
+
+    // column (a, b): interpolation, wJ and projection along t
+    if (act) {
+        long long *X = boxes + el * C::per, w[m];
+        const int kw = (int)(st[kFxW] >> 20) - 1022, bw = kw + 1022 + wab;
+        int far = 0, least = 0;
+        const double *we = wJ + (e0 + el) * MP + r;
+        const int up = fx30_up<N>(st);
+        fx_line<m, n, 1, oI>([&](int l) { return X[B2::at(a, b, l)] << up; },
+                             [&](int c, long long g) {
+                                 w[c] = fx30_mass(__ldg(we + c * mm), bw + c_fxd[N].wm[c], g, far, least);
+                             });
+        FxMost most;
+        fx_apply<n, m, 1, oIT>(w, [&](int l, long long y) {
+            X[B2::at(a, b, l)] = y;
+            most.see(y);
+        });
+        fx_element_max<mm>(st + kFxT1, (unsigned)most.value());
+        if (least < 0 || far > kFxRange || kw > 800 || kw < -800 || kq + kw > 800 || kq + kw < -800) st[kFxLeft1] = 1;
+    }
+    __syncthreads();
+
+    // projection along s and r
+    fx30_project_s<N, EPB_, B1, B2>(nel, boxes, boxes + C::SA, C::per, stats, kFxT1);
+    __syncthreads();
+    fx30_project_r<N, EPB_, B1>(
+        nel, boxes + C::SA, C::per, stats, kFxT1, kFxLeft1, [&](int e) { return fx1_exponent<N>(stats + e * K); },
+        [&](int e, int t, int l, double w) { Mq[(e0 + e) * NP + t * n + l] = w; });
+    for (int e = 0; e < nel; e++)
+        if (stats[e * K + kFxLeft1] != 0)  // the same for every thread
+            bp1_element64(reinterpret_cast<double *>(smem_raw), n, oI, oIT, wJ + (e0 + e) * MP, q + (e0 + e) * NP,
+                          Mq + (e0 + e) * NP);
+}
+
+// ---------------------------------------------------------------- BP3.0
+
+// Shared memory of EPB elements: four m^3 boxes, a word per line, the
+// statistics.
+template <int N, int EPB_>
+struct Fx30Layout {
+    static constexpr int n = N + 1, m = N + 2, nn = n * n, mm = m * m, NP = nn * n, MP = mm * m, EPB = EPB_;
+    using B0 = Box<n, n, n>;
+    using B1 = Box<m, n, n>;
+    using B2 = Box<m, m, n>;
+    using B3 = Box<m, m, m>;
+    static constexpr int S = B3::size, per = 4 * S;
+    static constexpr int threads = ((mm * EPB + 31) / 32) * 32;
+    static constexpr int off_e = EPB * per * 8;
+    static constexpr int off_s = off_e + EPB * 3 * mm * 4;
+    static constexpr int smem_ = off_s + EPB * kFx30Stats * 4;
+    static constexpr int smem = smem_ > threads * 8 ? smem_ : threads * 8;
+};
+
+// BP3.0 of elements [e0, e0 + nel) by the whole block (blockDim.x >=
+// Layout::threads); MASS: BP1.0 too, to Mq, with wJ the seventh factor.  PCG
+// as bp35_block.
+template <int N, int EPB_, bool PCG, bool MASS>
+__device__ __forceinline__ void bp30_fx_block(unsigned char *smem_raw, int64_t e0, int nel, const double *__restrict__ G,
+                                              double lambda, const double *__restrict__ q, double *__restrict__ Aq,
+                                              double *__restrict__ Mq, const double *__restrict__ z, double *p,
+                                              const double *__restrict__ beta, double *__restrict__ part_out) {
+    using C = Fx30Layout<N, EPB_>;
+    using B0 = typename C::B0;
+    using B1 = typename C::B1;
+    using B2 = typename C::B2;
+    using B3 = typename C::B3;
+    constexpr int n = C::n, m = C::m, nn = C::nn, mm = C::mm, NP = C::NP, MP = C::MP, S = C::S, K = kFx30Stats, QB = kFxBits30, qb = fx_qbits30(N);
+    constexpr int oI = fold_offset(N, kFoldI), oIT = fold_offset(N, kFoldIT);
+    constexpr int oDt = fold_offset(N, kFoldDt), oDtT = fold_offset(N, kFoldDtT);
+    const int el = threadIdx.x / mm, r = threadIdx.x - el * mm;
+    const bool act = el < nel;
+    const int u = r % m, v = r / m;
+    long long *boxes = reinterpret_cast<long long *>(smem_raw);
+    long long *A = boxes + el * C::per, *B = A + S, *Cx = B + S, *D = Cx + S;
+    int *ln = reinterpret_cast<int *>(smem_raw + C::off_e) + el * 3 * mm;
+    unsigned *stats = reinterpret_cast<unsigned *>(smem_raw + C::off_s), *st = stats + el * K;
+    if (threadIdx.x == 0) prefetch_l2(G + e0 * 7 * MP, (long long)nel * 7 * MP * 8);
+    for (int t = threadIdx.x; t < EPB_ * K; t += blockDim.x) stats[t] = 0;
+    __syncthreads();
+
+    double qv[n];
+    const bool col = act && r < nn;
+    if (col) fx30_load<N, PCG>(qv, (e0 + el) * NP + r, r, q, z, p, beta, st);
+    __syncthreads();
+    int kq = 0;
+    if (act) {
+        bool left;
+        kq = fx30_scale<N>(st, &left);
+        if (col) {
+#pragma unroll
+            for (int k = 0; k < n; k++) {
+                const int e = (__double2hiint(qv[k]) >> 20) & 0x7ff;
+                left = left || (kq == 0 && e == 0 && (fx_abs_hi(qv[k]) | __double2loint(qv[k])) != 0);
+                B[B0::at(r % n, r / n, k)] = fx_from_double<qb>(qv[k], kq + 1022 - e);
+            }
+        }
+        if (left) st[kFxLeft1] = st[kFxLeft30] = 1;
+    }
+    __syncthreads();
+
+    // interpolation along r (B -> C), s (C -> B) and t (B -> A)
+    for_tasks<nn, EPB_>(nel, [&](int e, int t) {
+        const long long *X = boxes + e * C::per + S;
+        long long *Y = boxes + e * C::per + 2 * S;
+        const int j = t % n, k = t / n;
+        fx_line<m, n, 1, oI>([&](int l) { return X[B0::at(l, j, k)]; }, [&](int l, long long y) { Y[B1::at(l, j, k)] = y; });
+    });
+    __syncthreads();
+    for_tasks<m * n, EPB_>(nel, [&](int e, int t) {
+        const long long *Y = boxes + e * C::per + 2 * S;
+        long long *X = boxes + e * C::per + S;
+        const int i = t % m, k = t / m;
+        FxMost most;
+        fx_line<m, n, 1, oI>([&](int l) { return Y[B1::at(i, l, k)]; },
+                             [&](int l, long long y) {
+                                 X[B2::at(i, l, k)] = y;
+                                 most.see(y);
+                             });
+        atomicMax(stats + e * K + kFxI, (unsigned)most.value());
+    });
+    __syncthreads();
+    const double *Ge = G + (e0 + el) * 7 * MP + r;
+    const int wuv = act ? c_fxd[N].wm[u] + c_fxd[N].wm[v] : 0;
+    int t3 = 3 * c_fxd[N].tau[kFoldI];  // exponent of the interpolated field over q's
+    if (act) {
+        t3 -= fx30_up<N>(st);
+        const int up = fx30_up<N>(st);
+        fx_line<m, n, 1, oI>([&](int l) { return B[B2::at(u, v, l)] << up; },
+                             [&](int l, long long y) { A[B3::at(u, v, l)] = y; });
+        fx30_scan<N, 4>(Ge, {6, 0, 3, 5}, wuv, st + kFxW);
+    }
+    __syncthreads();
+    const int kw = act ? (int)(st[kFxW] >> 20) - 1022 : 0;
+
+    // BP1.0: wJ and projection along t (A -> B), s (B -> C) and r (C -> Mq)
+    if constexpr (MASS) {
+        if (act) {
+            long long w[m];
+            const int bw = kw + 1022 + wuv;
+            int far = 0, least = 0;
+#pragma unroll
+            for (int c = 0; c < m; c++)
+                w[c] = fx30_mass(__ldg(Ge + 6 * MP + c * mm), bw + c_fxd[N].wm[c], A[B3::at(u, v, c)], far, least);
+            FxMost most;
+            fx_apply<n, m, 1, oIT>(w, [&](int l, long long y) {
+                B[B2::at(u, v, l)] = y;
+                most.see(y);
+            });
+            fx_element_max<mm>(st + kFxT1, (unsigned)most.value());
+            if (least < 0 || far > kFxRange || kw > 800 || kw < -800 || kq + kw > 800 || kq + kw < -800)
+                st[kFxLeft1] = 1;
+        }
+        __syncthreads();
+        fx30_project_s<N, EPB_, B1, B2>(nel, boxes + S, boxes + 2 * S, C::per, stats, kFxT1);
+        __syncthreads();
+        fx30_project_r<N, EPB_, B1>(
+            nel, boxes + 2 * S, C::per, stats, kFxT1, kFxLeft1, [&](int e) { return fx1_exponent<N>(stats + e * K); },
+            [&](int e, int t, int l, double w) { Mq[(e0 + e) * NP + t * n + l] = w; });
+        __syncthreads();
+    }
+
+    // derivatives along r (A -> B), s (A -> C) and t (A -> D)
+    if (act) {
+        int most = fx_derivative<B3, m, oDt, 0>(A, B, u, v);
+        most = max(most, fx_derivative<B3, m, oDt, 1>(A, Cx, u, v));
+        most = max(most, fx_derivative<B3, m, oDt, 2>(A, D, u, v));
+        fx_element_max<mm>(st + kFxU, (unsigned)most);
+    }
+    __syncthreads();
+
+    // chain rule at the points of column (a=u, b=v)
+    int basez = 0;
+    if (act) {
+        int kg = (int)(max(st[kFxG], max(st[kFxG + 1], st[kFxG + 2])) >> 20) - 1022;
+        bool left = kg > 800 || kg < -800 || kq + kg > 800 || kq + kg < -800;
+        const int sh = max(0, QB - 32 - fx_top((int)st[kFxU]));
+        basez = kq - qb + t3 + c_fxd[N].tau[kFoldDt] - sh + 2 + kg + c_fxd[N].tau[kFoldDtT];
+        const int eg = kg + 1022 + wuv;
+        FxRange range;
+#pragma unroll 4
+        for (int c = 0; c < m; c++) {
+            const int s = B3::at(u, v, c);
+            fx_chain(Ge + c * mm, MP, eg + c_fxd[N].wm[c], B[s] << sh, Cx[s] << sh, D[s] << sh, B[s], Cx[s], D[s], range);
+        }
+        if (left || range.left()) st[kFxLeft30] = 1;
+    }
+    __syncthreads();
+
+    // transposes, in place; ln: each line's scale
+    if (act) {
+        const int hr = fx_transpose<B3, m, oDtT, QB, 0>(B, u, v), hs = fx_transpose<B3, m, oDtT, QB, 1>(Cx, u, v),
+                  ht = fx_transpose<B3, m, oDtT, QB, 2>(D, u, v);
+        ln[r] = hr;
+        ln[mm + r] = hs;
+        ln[2 * mm + r] = ht;
+        fx_element_max<mm>(st + kFxH, (unsigned)(63 - __vimin3_s32(hr, hs, ht)));
+    }
+    __syncthreads();
+
+    // column: the three directions and lambda wJ q, aligned (-> D)
+    int zs = 0;
+    if (act) {
+        const int hm = 63 - (int)st[kFxH];  // every line is brought to the largest scale among them
+        basez -= hm;
+        int el2 = 0;  // |lambda| < 2^el2
+        if (lambda != 0.0) el2 = ((__double2hiint(lambda) >> 20) & 0x7ff) - 1022;
+        const int delta = kq - qb + t3 + kw + el2 - basez;  // scale of the mass term over the other's
+        zs = (lambda != 0.0) ? min(63, max(0, delta)) : 0;
+        const int ms = min(63, max(0, -delta)), bw = kw + el2 + 1022 + wuv, ht = ln[2 * mm + r] - hm + zs;
+        bool left = el2 > 200 || el2 < -200 || delta > 63 || kw > 800 || kw < -800 || kq + kw > 800 || kq + kw < -800;
+        if (lambda == 0.0) left = false;
+        FxMost most;
+        int far = 0, least = 0;
+#pragma unroll 4
+        for (int c = 0; c < m; c++) {
+            const int s = B3::at(u, v, c);
+            long long x = (B[s] >> min(63, ln[v + m * c] - hm + zs)) +
+                          (Cx[s] >> min(63, ln[mm + u + m * c] - hm + zs)) + (D[s] >> min(63, ht));
+            if (lambda != 0.0) {
+                const double wj = lambda * __ldg(Ge + 6 * MP + c * mm);
+                const int e = (__double2hiint(wj) >> 20) & 0x7ff, d = bw + c_fxd[N].wm[c] - e;
+                far = max(far, d);
+                least = min(least, d);
+                int gh, gl;
+                fx_off_diagonal(wj, d, gh, gl);
+                x += fx_mul(gh, gl, A[s]) >> ms;
+            }
+            D[s] = x;
+            most.see(x);
+        }
+        fx_element_max<mm>(st + kFxX, (unsigned)most.value());
+        if (left || least < 0 || far > kFxRange + 2) st[kFxLeft30] = 1;
+    }
+    __syncthreads();
+
+    // projection along t (D in place), s (D -> C) and r (C -> Aq)
+    if (act) {
+        const int sx = QB - 32 - fx_top((int)st[kFxX]), up = max(0, sx), down = max(0, -sx);
+        FxMost most;
+        fx_line<n, m, 1, oIT>([&](int l) { return (D[B3::at(u, v, l)] << up) >> down; },
+                              [&](int l, long long y) {
+                                  D[B2::at(u, v, l)] = y;
+                                  most.see(y);
+                              });
+        fx_element_max<mm>(st + kFxT30, (unsigned)most.value());
+        if (r == 0) ln[0] = basez + zs - sx + 3 * c_fxd[N].tau[kFoldIT];  // (every line's scale has been read)
+    }
+    __syncthreads();
+    fx30_project_s<N, EPB_, B1, B2>(nel, boxes + 3 * S, boxes + 2 * S, C::per, stats, kFxT30);
+    __syncthreads();
+    double dot = 0.0;  // p . Ap of the thread's lines
+    fx30_project_r<N, EPB_, B1>(
+        nel, boxes + 2 * S, C::per, stats, kFxT30, kFxLeft30,
+        [&](int e) { return reinterpret_cast<const int *>(smem_raw + C::off_e)[e * 3 * mm]; },
+        [&](int e, int t, int l, double w) {
+            const int64_t g = (e0 + e) * NP + t * n + l;
+            Aq[g] = w;
+            if (PCG) dot = fma(p[g], w, dot);
+        });
+    for (int e = 0; e < nel; e++) {  // (the conditions are the same for every thread)
+        const int64_t g0 = (e0 + e) * NP;
+        const double *qe = (PCG ? p : q) + g0, *ge = G + (e0 + e) * 7 * MP;
+        if (MASS && stats[e * K + kFxLeft1] != 0)
+            bp1_element64(reinterpret_cast<double *>(smem_raw), n, oI, oIT, ge + 6 * MP, qe, Mq + g0);
+        if (stats[e * K + kFxLeft30] != 0) {
+            bp30_element64(reinterpret_cast<double *>(smem_raw), n, oI, oIT, oDt, oDtT, ge, lambda, qe, Aq + g0);
+            if (PCG) {
+                __syncthreads();  // (the element's output is there)
+                for (int t = threadIdx.x; t < NP; t += blockDim.x) dot = fma(qe[t], Aq[g0 + t], dot);
+            }
+        }
+    }
+    if (PCG) {
+        __syncthreads();  // the shared boxes are reused for the reduction
+        const double tot = block_sum(dot, reinterpret_cast<double *>(smem_raw));
+        if (threadIdx.x == 0) *part_out = tot;
+    }
+}
+
+}  // namespace
+}  // namespace fem

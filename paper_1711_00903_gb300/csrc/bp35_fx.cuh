@@ -37,13 +37,10 @@
 
 #include "bp35_body.cuh"  // Bp35Layout
 #include "fx.cuh"
+#include "fx_point.cuh"
 
 namespace fem {
 namespace {
-
-// How far (in bits) below its element's largest a node's largest line, or a
-// point's largest factor, may lie.
-constexpr int kFxRange = 6;
 
 template <int N, int EPB_>
 struct Fx35Layout : Bp35Layout<double, N, EPB_> {
@@ -103,77 +100,6 @@ __device__ __noinline__ double bp35_element64(double *smem, int n, int oD, int o
         }
     }
     return dot;
-}
-
-// Balanced halves of a factor scaled to 62 bits; s as in fx_magnitude.  A
-// diagonal factor is positive (the element is left out otherwise).
-__device__ __forceinline__ void fx_diagonal(double g, int s, int &gh, int &gl) {
-    const long long m = (long long)fx_magnitude<62>(__double2hiint(g), (unsigned)__double2loint(g), s);
-    gh = fx_hi(m);
-    gl = fx_lo(m);
-}
-__device__ __forceinline__ void fx_off_diagonal(double g, int s, int &gh, int &gl) {
-    const int sg = __double2hiint(g) >> 31;  // 0, or -1: negates the halves (the low one to within a unit, 2^-62)
-    const long long m = (long long)fx_magnitude<62>(__double2hiint(g), (unsigned)__double2loint(g), s);
-    gh = fx_hi(m) * (sg | 1);
-    gl = fx_lo(m) ^ sg;
-}
-
-// (a x + b y + c z) / 2^64 of factors a, b, c below 2^62 (halves) and values
-// below 2^61: the cross products are summed apart, three of them reach 2^62.6.
-__device__ __forceinline__ long long fx_dot3(int ah, int al, long long x, int bh, int bl, long long y, int ch, int cl,
-                                             long long z) {
-    const int xh = fx_hi(x), xl = fx_lo(x), yh = fx_hi(y), yl = fx_lo(y), zh = fx_hi(z), zl = fx_lo(z);
-    const long long h = mad_wide(ch, zh, mad_wide(bh, yh, mul_wide(ah, xh)));
-    const long long m = mad_wide(ch, zl, mad_wide(bh, yl, mul_wide(ah, xl)));
-    const long long l = mad_wide(cl, zh, mad_wide(bl, yh, mul_wide(al, xh)));
-    return h + (long long)(int)(m >> 32) + (long long)(int)(l >> 32);
-}
-
-// Point l of the line of direction D at (u, v) in an element box (0: r at
-// (j=u, k=v), 1: s at (i=u, k=v), 2: t at (i=u, j=v)).
-template <class B, int D>
-__device__ __forceinline__ int fx_at(int l, int u, int v) {
-    return D == 0 ? B::at(l, u, v) : D == 1 ? B::at(u, l, v) : B::at(u, v, l);
-}
-
-// The derivatives along the lines of direction D from one box to another (or
-// in place); returns the largest |high word| of the results, *field that of
-// the line.
-template <class B, int n, int OFF, int D>
-__device__ __forceinline__ int fx_derivative(const long long *from, long long *to, int u, int v, int *field) {
-    long long x[n];
-#pragma unroll
-    for (int l = 0; l < n; l++) x[l] = from[fx_at<B, D>(l, u, v)];
-    int f = fx_line_max(x);
-    if (f == 0) {  // below 2^32: tell a line of zeros from a line of small values
-        int any = 0;
-#pragma unroll
-        for (int l = 0; l < n; l++) any |= (int)x[l];
-        f = any != 0;
-    }
-    *field = f;
-    int hi = 0, lo = 0;
-    fx_apply<n, n, -1, OFF>(x, [&](int l, long long y) {
-        to[fx_at<B, D>(l, u, v)] = y;
-        hi = max(hi, (int)(y >> 32));
-        lo = min(lo, (int)(y >> 32));
-    });
-    return max(hi, ~lo);
-}
-
-// The transpose along a line of direction D, in place, the line first scaled
-// up to QB bits; returns the shift.
-template <class B, int n, int OFF, int QB, int D>
-__device__ __forceinline__ int fx_transpose(long long *box, int u, int v) {
-    long long x[n];
-#pragma unroll
-    for (int l = 0; l < n; l++) x[l] = box[fx_at<B, D>(l, u, v)];
-    const int h = max(0, QB - 32 - fx_top(fx_line_max(x)));
-#pragma unroll
-    for (int l = 0; l < n; l++) x[l] <<= h;
-    fx_apply<n, n, -1, OFF>(x, [&](int l, long long y) { box[fx_at<B, D>(l, u, v)] = y; });
-    return h;
 }
 
 // Whether node (i, j, k), none of whose lines reaches the element's scale, is
@@ -277,12 +203,12 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
     // box 0; ln: each line's largest value
     int m = 0;
     if (act) {
-        m = fx_derivative<B, n, oD, 0>(box, box + B::size, u, v, ln + r);
-        m = max(m, fx_derivative<B, n, oD, 1>(box, box + 2 * B::size, u, v, ln + nn + r));
+        m = fx_derivative<B, n, oD, 0, true>(box, box + B::size, u, v, ln + r);
+        m = max(m, fx_derivative<B, n, oD, 1, true>(box, box + 2 * B::size, u, v, ln + nn + r));
     }
     __syncthreads();
     if (act) {
-        m = max(m, fx_derivative<B, n, oD, 2>(box, box, u, v, ln + 2 * nn + r));
+        m = max(m, fx_derivative<B, n, oD, 2, true>(box, box, u, v, ln + 2 * nn + r));
         fx_element_max<nn>(st + 4, (unsigned)m);
         // the diagonal factors' largest exponents, without the weights
         // (prefetched into L2 when the block began)
@@ -319,33 +245,14 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
         const int sh = QB - 32 - fx_top((int)st[4]);
         base = kq - qb + c_fxd[N].tau[kFoldD] - sh + 2 + kg + c_fxd[N].tau[kFoldDT];
         const int eg = kg + 1022 + wuv;
-        int smin = 0, far = 0, neg = 0;
+        FxRange range;
 #pragma unroll(UC)
         for (int k = 0; k < n; k++) {
             const int s = B::at(u, v, k);
-            double g[6];
-#pragma unroll
-            for (int h = 0; h < 6; h++) g[h] = __ldg(Ge + h * NP + k * nn);
-            const int bk = eg + c_fxd[N].wn[k];
-            neg |= __double2hiint(g[0]) | __double2hiint(g[3]) | __double2hiint(g[5]);
-            const int s0 = bk - (__double2hiint(g[0]) >> 20), s3 = bk - (__double2hiint(g[3]) >> 20),
-                      s5 = bk - (__double2hiint(g[5]) >> 20), s1 = bk - ((__double2hiint(g[1]) >> 20) & 0x7ff),
-                      s2 = bk - ((__double2hiint(g[2]) >> 20) & 0x7ff), s4 = bk - ((__double2hiint(g[4]) >> 20) & 0x7ff);
-            smin = __vimin3_s32(smin, __vimin3_s32(s0, s1, s2), __vimin3_s32(s3, s4, s5));
-            far = max(far, __vimin3_s32(s0, s3, s5));
-            int gh[6], gl[6];
-            fx_diagonal(g[0], s0, gh[0], gl[0]);
-            fx_off_diagonal(g[1], s1, gh[1], gl[1]);
-            fx_off_diagonal(g[2], s2, gh[2], gl[2]);
-            fx_diagonal(g[3], s3, gh[3], gl[3]);
-            fx_off_diagonal(g[4], s4, gh[4], gl[4]);
-            fx_diagonal(g[5], s5, gh[5], gl[5]);
-            const long long dr = box[B::size + s] << sh, ds = box[2 * B::size + s] << sh, dt = box[s] << sh;
-            box[B::size + s] = fx_dot3(gh[0], gl[0], dr, gh[1], gl[1], ds, gh[2], gl[2], dt);
-            box[2 * B::size + s] = fx_dot3(gh[1], gl[1], dr, gh[3], gl[3], ds, gh[4], gl[4], dt);
-            box[s] = fx_dot3(gh[2], gl[2], dr, gh[4], gl[4], ds, gh[5], gl[5], dt);
+            long long *rr = box + B::size + s, *ss = rr + B::size, *tt = box + s;
+            fx_chain(Ge + k * nn, NP, eg + c_fxd[N].wn[k], *rr << sh, *ss << sh, *tt << sh, *rr, *ss, *tt, range);
         }
-        if (bad || smin < 0 || far > kFxRange || neg < 0) st[5] = 1;
+        if (bad || range.left()) st[5] = 1;
     }
     __syncthreads();
 

@@ -72,6 +72,9 @@ cudaError_t prepare_bp35(int N, const double *fold_table);
 // FP64 BP3.5 (bp35_fx.cu): its preparation and its blocks (the PCG partials).
 cudaError_t prepare_bp35_fx(int N, const double *fold_table);
 int64_t bp35_fx_blocks(int N, int64_t E);
+// FP64 BP3.0 and BP1.0 + BP3.0 (bp30_fx.cu).
+cudaError_t prepare_bp30_fx(int N, const double *fold_table);
+int64_t bp30_fx_blocks(int N, int64_t E);
 cudaError_t prepare_bp30(int N, const double *fold_table);
 cudaError_t launch_geofacs_gauss_pair(const fem_basis *b, int64_t E, const double *verts, double *G30, double *wJ,
                                       cudaStream_t s);

@@ -73,7 +73,7 @@ struct FxSum {
 
 // y (P) = A x (Q) along one line, A folded at table offset OFF with parity
 // SIG (eo.cuh), scaled by 2^-tau (FxDegree): |y| < 1.02 2^B for |x| < 2^B, B =
-// fx_bits35, fx_bits30.  put(a, y_a) takes each output as it is formed, so
+// fx_bits35, kFxBits30.  put(a, y_a) takes each output as it is formed, so
 // that a line needs the registers of its folded inputs and two sums only.
 template <int P, int Q, int SIG, int OFF, class F>
 __device__ __forceinline__ void fx_apply(const long long (&x)[Q], F &&put) {

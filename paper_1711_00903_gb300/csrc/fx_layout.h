@@ -23,11 +23,17 @@ struct FxTables {
 };
 
 // Bits of a value (|x| < 2^bits) at the input of a contraction, and of its
-// output: 61, and 60 where a sum of cross products of 61-bit values could
-// overflow (fx_tables() checks the sums of every row).  BP3.5 contracts lines
-// of n points (its first contraction takes 60 bits), BP1.0 and BP3.0 up to m.
+// output: 61 and 60, as the sums of cross products of every row allow
+// (fx_tables() checks them, for BP1.0 and BP3.0 with 8 % for what three
+// contractions in a row may add).  BP3.5's first contraction takes one bit
+// less than its second.
 __host__ __device__ constexpr int fx_bits35(int N) { return N >= 10 ? 60 : 61; }
-__host__ __device__ constexpr int fx_bits30(int N) { return N >= 6 ? 60 : 61; }
+constexpr int kFxBits30 = 60;
+// Bits of the field of BP1.0 and BP3.0: their interpolations are scaled by one
+// half, and a row's absolute sum is up to 2.43 (N = 15), so that from N = 7 on
+// (1.97) three in a row may grow by 1.8; at N = 15 the cross products need one
+// bit more.
+__host__ __device__ constexpr int fx_qbits30(int N) { return N == 15 ? 58 : N >= 7 ? 59 : 60; }
 
 // Built once; aborts nothing: a table that breaks a bound is reported by
 // fx_table_violations().

@@ -31,14 +31,19 @@ FxEntry halves(__int128 c, int *bad) {
     return e;
 }
 
-// Folds A (P x Q, row-major) scaled by 2^-tau into out; returns the number
+// Folds A (P x Q, row-major, parity sig) scaled by 2^-tau into out; returns the number
 // of bounds that do not hold.
-int fold_scaled(int P, int Q, const double *A, int bits, int tau, FxEntry *out) {
+int fold_scaled(int P, int Q, int sig, const double *A, int bits, double room, int tau, FxEntry *out) {
     int bad = 0;
     const int hp = P / 2, hq = Q / 2;
-    auto I = [&](int a, int i) { return scaled(A[a * Q + i], tau); };
+    // the entry with its image under the operator's symmetry: the mean of the
+    // two is nearer to the exact entry than either
+    auto I = [&](int a, int i) {
+        const __int128 x = scaled(A[a * Q + i], tau), y = scaled(A[(P - 1 - a) * Q + (Q - 1 - i)], tau);
+        return (x + (sig > 0 ? y : -y)) >> 1;
+    };
     FxEntry *S = out, *T = out + hp * hq, *cm = T + hp * hq, *rm = cm + (Q % 2 ? hp : 0);
-    // bounds of a row's sums, with |e| <= 2^(bits + 1): the sum of the high
+    // bounds of a row's sums, with |e| <= room 2^(bits + 1): the sum of the high
     // products and that of the cross products below 2^63
     auto check = [&](const FxEntry *r, int n, const FxEntry *extra) {
         double h = 0.0, l = 0.0;
@@ -50,7 +55,7 @@ int fold_scaled(int P, int Q, const double *A, int bits, int tau, FxEntry *out) 
             h += std::fabs((double)extra->h);
             l += std::fabs((double)extra->l);
         }
-        const double xh = std::ldexp(1.0, bits + 1 - 32) + 1.0, lim = std::ldexp(1.0, 63) - std::ldexp(1.0, 32);
+        const double xh = room * std::ldexp(1.0, bits + 1 - 32), lim = std::ldexp(1.0, 63) - std::ldexp(1.0, 32);
         if (h * xh >= lim || h * std::ldexp(1.0, 31) + l * xh >= lim) bad++;
     };
     for (int a = 0; a < hp; a++)
@@ -72,20 +77,24 @@ int fold_scaled(int P, int Q, const double *A, int bits, int tau, FxEntry *out) 
     return bad;
 }
 
-// The smallest tau whose scaled rows hold the bounds: a row's absolute sum
-// at most 2^tau, up to 2 % over (the outputs have that room), every entry's
-// high half within 32 bits.
-int fold(int P, int Q, const double *A, int bits, FxEntry *out) {
+// At kAutoTau, the smallest tau whose scaled rows hold the bounds: a row's
+// absolute sum at most 2^tau, up to 2 % over (the outputs have that room),
+// every entry's high half within 32 bits.
+constexpr int kAutoTau = -1;
+int fold(int P, int Q, int sig, const double *A, int bits, double room, int tau, FxEntry *out) {
+    if (tau != kAutoTau) {
+        g_violations += fold_scaled(P, Q, sig, A, bits, room, tau, out);
+        return tau;
+    }
     double nu = 0.0;
     for (int a = 0; a < P; a++) {
         double s = 0.0;
         for (int i = 0; i < Q; i++) s += std::fabs(A[a * Q + i]);
         nu = s > nu ? s : nu;
     }
-    int tau;
     std::frexp(nu / 1.02, &tau);
-    int bad = fold_scaled(P, Q, A, bits, tau, out);
-    for (int up = 0; bad && up < 2; up++) bad = fold_scaled(P, Q, A, bits, ++tau, out);
+    int bad = fold_scaled(P, Q, sig, A, bits, room, tau, out);
+    for (int up = 0; bad && up < 2; up++) bad = fold_scaled(P, Q, sig, A, bits, room, ++tau, out);
     g_violations += bad;
     return tau;
 }
@@ -115,11 +124,18 @@ const FxTables &fx_tables() {
                 for (int b = 0; b < m; b++) DtT[b * m + a] = std::ldexp(hb.Dt[a * m + b], d.wm[a] - d.wm[b]);
             const double *ops[kFoldCount] = {hb.I, IT, hb.D, DT, hb.Dt, DtT};
             for (int op = 0; op < kFoldCount; op++)
-                d.tau[op] = fold(fold_rows(op, n, m), fold_cols(op, n, m), ops[op],
-                                 op == kFoldD    ? fx_bits35(N) - 1
-                                 : op == kFoldDT ? fx_bits35(N)
-                                                 : fx_bits30(N),
-                                 t->c + fold_offset(N, op));
+                d.tau[op] =
+                    op == kFoldI
+                        ? fold(m, n, 1, hb.I, fx_qbits30(N), N >= 7 ? 1.5 : 1.08, 1, t->c + fold_offset(N, op))
+                        : fold(fold_rows(op, n, m), fold_cols(op, n, m), op == kFoldIT ? 1 : -1, ops[op],
+                               op == kFoldD    ? fx_bits35(N) - 1
+                               : op == kFoldDT ? fx_bits35(N)
+                               : op == kFoldDt ? fx_qbits30(N)
+                                               : kFxBits30,
+                               op == kFoldDt   ? (N >= 7 ? 1.25 : 1.0)
+                               : op == kFoldIT ? 1.08
+                                               : 1.0,
+                               kAutoTau, t->c + fold_offset(N, op));
         }
     });
     return *t;

@@ -8,8 +8,9 @@ Bar: |y - y_oracle| <= 8 (1.5 n + 17) 2^-53 b, with b the same operator on
 absolute values and on operators folded even-odd as FP64 lines evaluate them,
 (|A[a][i]| + |A[a][Q-1-i]|) for A[a][i]: an FP64 evaluation makes at most
 about n/2 + 3 roundings per contraction on the longest chain (three
-contractions in BP3.5), 8 in the chain rule and the sums, for each side,
-times 4 for what the two evaluations order differently."""
+contractions in BP3.5, six in BP1.0, nine in BP3.0: 1.5 n, 3 n, 4.5 n), 8 in
+the chain rule and the sums, for each side, times 4 for what the two
+evaluations order differently."""
 import numpy as np
 import pytest
 
@@ -76,7 +77,56 @@ class Op:
         return 8 * (self.chain * self.n + 17) * 2.0 ** -53
 
 
-OPS = {"bp35": Op}
+class Dealiased(Op):
+    """BP3.0: nine contractions on the longest chain."""
+
+    chain = 4.5
+
+    def factors(self, verts):
+        return oracle.geofacs(self.N, 3, verts)[0]
+
+    def oracle(self, geo, q):
+        return oracle.bp30(self.N, geo, 0.37, q)
+
+    def apply(self, geo, q):
+        fem = _fem()
+        return fem.fem_bp30_apply(fem.fem_basis_setup(self.N), _dev(geo), 0.37, _dev(q)).cpu().numpy()
+
+    def _interp(self, q):
+        u, I = np.abs(q).reshape(-1, self.n, self.n, self.n), _folded_abs(self.b.I)
+        return _along(I, _along(I, _along(I, u, 3), 2), 1)
+
+    def _project(self, g, shape):
+        IT = _folded_abs(self.b.I.T)
+        return _along(IT, _along(IT, _along(IT, g, 3), 2), 1).reshape(shape)
+
+    def bound(self, geo, q):
+        u = self._interp(q)
+        s, wj = _stiff_abs(self.b.Dt, geo, u)
+        return self._project(s + 0.37 * wj * u, q.shape)
+
+
+class Mass(Dealiased):
+    """BP1.0: six contractions; its factors are the seventh plane."""
+
+    chain = 3.0
+
+    def factors(self, verts):
+        return oracle.geofacs(self.N, 1, verts)[0]
+
+    def oracle(self, geo, q):
+        return oracle.bp1(self.N, geo, q)
+
+    def apply(self, geo, q):
+        fem = _fem()
+        return fem.fem_bp1_apply(fem.fem_basis_setup(self.N), _dev(geo), _dev(q)).cpu().numpy()
+
+    def bound(self, geo, q):
+        u = self._interp(q)
+        return self._project(np.abs(geo).reshape(u.shape) * u, q.shape)
+
+
+OPS = {"bp35": Op, "bp30": Dealiased, "bp1": Mass}
 
 
 def _check(op, geo, q):
@@ -119,6 +169,17 @@ def test_elements_of_every_kind(name, N):
     # an element's result does not depend on its neighbours in the block
     for e in (0, 3, 10):
         np.testing.assert_array_equal(op.apply(geo[e:e + 1], q[e:e + 1])[0], got[e])
+
+
+@pytest.mark.parametrize("N", range(1, 16))
+def test_one_pass_is_both_operators(N):
+    """BP1.0 and BP3.0 in one pass: the bits of each alone, whichever path an element takes."""
+    op, mass = Dealiased(N), Mass(N)
+    geo, q = _elements(op)
+    fem = _fem()
+    m, a = fem.fem_bp1_bp30_apply(fem.fem_basis_setup(N), _dev(geo), 0.37, _dev(q))
+    np.testing.assert_array_equal(a.cpu().numpy(), op.apply(geo, q))
+    np.testing.assert_array_equal(m.cpu().numpy(), mass.apply(np.ascontiguousarray(geo[:, 6]), q))
 
 
 @pytest.mark.parametrize("name", sorted(OPS))
