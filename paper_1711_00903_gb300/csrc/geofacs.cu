@@ -4,15 +4,30 @@
 // planes Grr, Grs, Grt, Gss, Gst, Gtt, wJ (BP3.5 at GLL nodes, BP3.0 at
 // Gauss points) or wJ alone (BP1.0 at Gauss points).
 //
-// GB300 design.  FP64-issue bound like the operators.  The columns of X of
-// a trilinear map factor over the tensor grid: dx/dr depends on (s, t) only,
-// dx/ds on (r, t) and dx/dt on (r, s), so each block first tabulates the
-// three q x q column tables of its element in shared memory (O(q^2) work),
-// then every point needs only the cofactor vectors C_r = X_s x X_t,
-// C_s = X_t x X_r, C_t = X_r x X_s (the rows of |J| X^{-1}), the
-// determinant X_r . C_r and the six products G = C C^T / |J|.  Stores are
-// coalesced per plane.
-#include "kernels_common.cuh"
+// GB300 design.  The columns of X of a trilinear map factor over the tensor
+// grid: dx/dr depends on (s, t) only, dx/ds on (r, t) and dx/dt on (r, s), so
+// each block first tabulates the three q x q column tables of its element in
+// shared memory (O(q^2) work), then every point needs only the cofactor
+// vectors C_r = X_s x X_t, C_s = X_t x X_r, C_t = X_r x X_s (the rows of |J|
+// X^{-1}), the determinant X_r . C_r and the six products G = C C^T / |J|.
+// Stores are coalesced per plane.
+//
+// In FP64 that is 52 instructions a point at 2 per clock and SM.  The point
+// work therefore runs on the integer multiply-add pipe (fx.cuh) in 62-bit
+// fixed point, one scale for each of X_r, X_s, X_t of an element; the result
+// is converted to FP64 once.  All factors of 32^3 elements at N = 7: 1315 us
+// against 4186 in FP64; the bound is the integer multiply-adds (about 150 a
+// point, half their rate) and the seven conversions on the FP64 pipe.  The
+// error against quadruple precision is 0.55 to 0.83 of the FP64 kernel's over
+// all planes, 0.7 to 1 plane by plane on a 10 % jittered mesh.
+//
+// An element for which a scale does not serve is computed in FP64: a component of a column that is far below the
+// column's largest but not zero (a slightly skewed element, whose small
+// off-diagonal factors FP64 gives to full relative accuracy), a determinant
+// that is not positive, extreme or non-finite vertices.  The choice is made
+// element by element.
+#define FEM_FX_TABLES
+#include "fx.cuh"
 
 namespace fem {
 namespace {
@@ -20,12 +35,14 @@ namespace {
 template <int qn>
 struct GeoCfg {
     static constexpr int QP = qn * qn * qn, qq = qn * qn;
-    static constexpr int SD = (qq > 36) ? qq : 36;  // per-thread minima, or the 36 map coefficients
-    static constexpr int smem_elem = (24 + 9 * qq + SD) * 8;
-    // about 512 threads per block (measured faster than 256 and 128 at N = 7)
-    static constexpr int EPB = pick_epb(qn, smem_elem, 512);
+    static constexpr int SD = qq + 4;  // per-thread minima; three scales and what is left to FP64 (eight words)
+    static constexpr int PER = pad2(24 + 36 + 9 * qq + SD);  // vertices, map coefficients, tables, minima
+    static constexpr int smem_elem = PER * 8;
+    // about 256 threads per block: with four resident blocks 1315 us for all
+    // factors at N = 7 on 32^3 elements, against 1396 with two of 512
+    static constexpr int EPB = pick_epb(qn, smem_elem, 256);
     static constexpr int threads = qq * EPB;
-    static constexpr int smem = (2 * pad2(qn) + EPB * pad2(24 + 9 * qq + SD)) * 8;
+    static constexpr int smem = (4 * pad2(qn) + EPB * PER) * 8;
 };
 
 // 1 / d in FP64: an FP32 reciprocal seed refined by two Newton steps
@@ -54,6 +71,50 @@ __device__ __forceinline__ double recip(double d) {
     return fma(r, e, r);
 }
 
+// a b / 2^(64 - k) of values up to 2^62 (the result below 2^63); k <= 3.
+template <int k>
+__device__ __forceinline__ long long geo_mul(long long a, long long b) {
+    const int ah = fx_hi(a), al = fx_lo(a), bh = fx_hi(b), bl = fx_lo(b);
+    const long long m = mad_wide(ah, bl, mad_wide(al, bh, 1ll << (31 - k)));
+    return (mul_wide(ah, bh) << k) + (m >> (32 - k));
+}
+// a b - c d over 2^64.
+__device__ __forceinline__ long long geo_cross(long long a, long long b, long long c, long long d) {
+    return geo_mul<0>(a, b) - geo_mul<0>(c, d);
+}
+// a . b over 2^(64 - k) of vectors below 2^62, exact to the last unit when
+// below 2^63.
+template <int k>
+__device__ __forceinline__ long long geo_dot(const long long (&a)[3], const long long (&b)[3]) {
+    long long h = 0, m = 0;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const int ah = fx_hi(a[d]), al = fx_lo(a[d]), bh = fx_hi(b[d]), bl = fx_lo(b[d]);
+        h = d == 0 ? mul_wide(ah, bh) : mad_wide(ah, bh, h);
+        m += mad_wide(ah, bl, mad_wide(al, bh, 1ll << (31 - k))) >> (32 - k);
+    }
+    return (h << k) + m;
+}
+
+// 2^122 / d for 2^61 <= d < 2^62: a binary32 reciprocal seed and two Newton
+// steps r <- r + r (1 - d r), to about 2^-57.
+__device__ __forceinline__ long long geo_recip(long long d) {
+    const float x = __uint_as_float(0x3f000000u | ((unsigned)(d >> 38) & 0x7fffffu));  // d / 2^62
+    const unsigned rb = min(__float_as_uint(__frcp_rn(x)), 0x3fffffffu);               // (1, 2)
+    long long r = (long long)((rb & 0x7fffffu) | 0x800000u) << 37;
+#pragma unroll
+    for (int it = 0; it < 2; it++) r += geo_mul<0>(r, ((1ll << 58) - geo_mul<0>(d, r)) << 6);
+    return r;
+}
+
+// x 2^(62 - k) for |x| < 2^k, as an integer.
+__device__ __forceinline__ long long geo_fixed(double x, int k) {
+    return fx_from_double<62>(x, k + 1022 - ((__double2hiint(x) >> 20) & 0x7ff));
+}
+
+// A component of a column may lie this many bits below the column's largest.
+constexpr int kGeoRange = 6;
+
 // kind: 1 = wJ only, 2 and 3 = 7 planes, 4 = 7 planes and, in wj2, a copy
 // of the wJ plane in the BP1.0 layout (BP3.0 and BP1.0 factors live at the
 // same Gauss points, so one pass serves both); MIN: also the per-element
@@ -64,14 +125,17 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
                                              double *__restrict__ geo, double *__restrict__ detJ_min,
                                              double *__restrict__ wj2) {
     using C = GeoCfg<qn>;
-    constexpr int QP = C::QP, qq = C::qq, EPB = C::EPB;
-    constexpr int PER = pad2(24 + 9 * qq + C::SD);
+    constexpr int QP = C::QP, qq = C::qq, EPB = C::EPB, PER = C::PER;
     extern __shared__ double smem[];
     double *sx = smem, *sw = sx + pad2(qn);
-    double *buf = sw + pad2(qn);
+    long long *fx = reinterpret_cast<long long *>(sw + pad2(qn)), *fw = fx + pad2(qn);  // nodes, weights in 62 bits
+    double *buf = reinterpret_cast<double *>(fw + pad2(qn));
     for (int t = threadIdx.x; t < qn; t += blockDim.x) {
+        const double w = __ldg(weights + t);
         sx[t] = __ldg(nodes + t);
-        sw[t] = __ldg(weights + t);
+        sw[t] = w;
+        fx[t] = __double2ll_rn(sx[t] * 0x1p62);
+        fw[t] = geo_fixed(w, (__double2hiint(w) >> 20) - 1022);
     }
     const int64_t e0 = (int64_t)blockIdx.x * EPB;
     const int64_t nel = (E - e0) < EPB ? (E - e0) : EPB;
@@ -85,11 +149,13 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
     const int u = ab % qn, v = ab / qn;
     const bool valid = el < nel;
     const int64_t e = e0 + el;
-    const double *vx = buf + el * PER;     // vertices [c][d]
-    double *Xr = buf + el * PER + 24;      // dx/dr at (s_u, t_v): [u][v][d]
-    double *Xs = Xr + 3 * qq;              // dx/ds at (r_u, t_v)
-    double *Xt = Xs + 3 * qq;              // dx/dt at (r_u, s_v)
-    double *sdet = Xt + 3 * qq;            // per-thread minimum |J|
+    const double *vx = buf + el * PER;  // vertices [c][d]
+    double *K = buf + el * PER + 24;    // 36 map coefficients
+    double *Xr = K + 36;                // dx/dr at (s_u, t_v): [u][v][d]
+    double *Xs = Xr + 3 * qq;           // dx/ds at (r_u, t_v)
+    double *Xt = Xs + 3 * qq;           // dx/dt at (r_u, s_v)
+    double *sdet = Xt + 3 * qq;         // per-thread minimum |J|
+    int *scale = reinterpret_cast<int *>(sdet + qq);  // |X_dir| < 2^scale[dir]; [4..6]: the element is left to FP64; [7]: G is
 
     // tabulate the three column tables of X.  Along r the map's derivative is
     // dx/dr(s, t) = 1/8 [ A (1-s)(1-t) + B (1+s)(1-t) + C (1-s)(1+t) + D (1+s)(1+t) ]
@@ -98,7 +164,6 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
     // holds along s and t with their own edges.  The 3 x 4 x 3 coefficients
     // of an element are formed once (in shared memory), then each table entry
     // costs three FMAs per component.
-    double *K = sdet;  // 36 coefficients, reused below for the minimum
     for (int ci = ab; ci < 36; ci += qq) {
         // K[(dir*4 + w)*3 + d]: dir 0 = r, 1 = s, 2 = t; w = coefficient
         const int dir = ci / 12, w = (ci / 3) % 4, d = ci % 3;
@@ -126,17 +191,41 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
         K[ci] = 0.125 * kv;
     }
     __syncthreads();
-    {
-        // entry (u, v): X_r at (s_u, t_v), X_s at (r_u, t_v), X_t at (r_u, s_v)
-        const double p = sx[u], w2 = sx[v];
+    // scales: a column's entries are bounded by the sum of its coefficients
+    for (int d = ab; d < 3; d += qq) {
+        int most = 0, e3[3];
+        bool left = false;
 #pragma unroll
-        for (int d = 0; d < 3; d++) {
-            Xr[ab * 3 + d] = fma(w2, fma(p, K[(0 * 4 + 3) * 3 + d], K[(0 * 4 + 2) * 3 + d]),
-                                 fma(p, K[(0 * 4 + 1) * 3 + d], K[(0 * 4 + 0) * 3 + d]));
-            Xs[ab * 3 + d] = fma(w2, fma(p, K[(1 * 4 + 3) * 3 + d], K[(1 * 4 + 2) * 3 + d]),
-                                 fma(p, K[(1 * 4 + 1) * 3 + d], K[(1 * 4 + 0) * 3 + d]));
-            Xt[ab * 3 + d] = fma(w2, fma(p, K[(2 * 4 + 3) * 3 + d], K[(2 * 4 + 2) * 3 + d]),
-                                 fma(p, K[(2 * 4 + 1) * 3 + d], K[(2 * 4 + 0) * 3 + d]));
+        for (int c = 0; c < 3; c++) {
+            const double *k = K + d * 12 + c;
+            const double sum = fabs(k[0]) + fabs(k[3]) + fabs(k[6]) + fabs(k[9]);
+            e3[c] = sum == 0.0 ? -10000 : ((__double2hiint(sum) >> 20) & 0x7ff) - 1022;
+            most = c == 0 ? e3[0] : max(most, e3[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; c++) left = left || (e3[c] != -10000 && e3[c] < most - kGeoRange);
+        scale[d] = most;
+        if (d == 0) scale[7] = 0;
+        scale[4 + d] = left || most > 150 || most < -150;
+    }
+    __syncthreads();
+    const int kr = scale[0], ks = scale[1], kt = scale[2];
+    bool left = scale[4] | scale[5] | scale[6];
+    long long *Fr = reinterpret_cast<long long *>(Xr), *Fs = reinterpret_cast<long long *>(Xs),
+              *Ft = reinterpret_cast<long long *>(Xt);
+    if (!left) {
+        // entry (u, v): X_r at (s_u, t_v), X_s at (r_u, t_v), X_t at (r_u, s_v)
+        const long long p = fx[u], w2 = fx[v];
+#pragma unroll
+        for (int dir = 0; dir < 3; dir++) {
+            const int k = dir == 0 ? kr : dir == 1 ? ks : kt;
+            long long *F = dir == 0 ? Fr : dir == 1 ? Fs : Ft;
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                const double *kk = K + dir * 12 + d;
+                F[ab * 3 + d] = geo_fixed(kk[0], k) + geo_mul<2>(p, geo_fixed(kk[3], k)) +
+                                geo_mul<2>(w2, geo_fixed(kk[6], k) + geo_mul<2>(p, geo_fixed(kk[9], k)));
+            }
         }
     }
     __syncthreads();
@@ -144,46 +233,129 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
     // thread (a, b) = (u, v) walks the c direction
     const int a = u, b = v;
     const double wab = sw[a] * sw[b];
-    double xt[3];
-#pragma unroll
-    for (int d = 0; d < 3; d++) xt[d] = Xt[(a + qn * b) * 3 + d];  // dx/dt at (r_a, s_b)
     double mindet = 1e300;
     double *ge = geo + (valid ? e : 0) * (kind == 1 ? 1 : 7) * (int64_t)QP + ab;
-#pragma unroll 1
-    for (int c = 0; c < qn; c++) {
-        double xr[3], xs[3];
+    if (valid && !left) {
+        long long xt[3];
 #pragma unroll
-        for (int d = 0; d < 3; d++) {
-            xr[d] = Xr[(b + qn * c) * 3 + d];  // dx/dr at (s_b, t_c)
-            xs[d] = Xs[(a + qn * c) * 3 + d];  // dx/ds at (r_a, t_c)
-        }
-        // C_r = X_s x X_t
-        const double Cr0 = xs[1] * xt[2] - xs[2] * xt[1];
-        const double Cr1 = xs[2] * xt[0] - xs[0] * xt[2];
-        const double Cr2 = xs[0] * xt[1] - xs[1] * xt[0];
-        const double det = xr[0] * Cr0 + xr[1] * Cr1 + xr[2] * Cr2;
-        const double W = wab * sw[c];
-        if (MIN) mindet = fmin(mindet, det);
-        if (kind == 1) {
-            if (valid) ge[c * qq] = W * det;
-        } else {
-            const double Cs0 = xt[1] * xr[2] - xt[2] * xr[1];
-            const double Cs1 = xt[2] * xr[0] - xt[0] * xr[2];
-            const double Cs2 = xt[0] * xr[1] - xt[1] * xr[0];
-            const double Ct0 = xr[1] * xs[2] - xr[2] * xs[1];
-            const double Ct1 = xr[2] * xs[0] - xr[0] * xs[2];
-            const double Ct2 = xr[0] * xs[1] - xr[1] * xs[0];
-            const double f = W * recip(det);
-            if (valid) {
+        for (int d = 0; d < 3; d++) xt[d] = Ft[(a + qn * b) * 3 + d];  // dx/dt at (r_a, s_b)
+        // the weights' product, its leading bit at 61
+        long long w2 = geo_mul<2>(fw[a], fw[b]);
+        int kw = (__double2hiint(sw[a]) >> 20) + (__double2hiint(sw[b]) >> 20) - 2 * 1022;
+        const int lead = __clzll(w2) - 2;
+        w2 <<= lead;
+        kw -= lead;
+        const int K3 = kr + ks + kt;
+        bool lost = false;  // a determinant that is not positive, or cancelled away
+        int most = 0;       // of the squares' high words: at 2^30 and above (long cofactors) they do not fit
+#pragma unroll 1
+        for (int c = 0; c < qn; c++) {
+            long long xr[3], xs[3];
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                xr[d] = Fr[(b + qn * c) * 3 + d];  // dx/dr at (s_b, t_c)
+                xs[d] = Fs[(a + qn * c) * 3 + d];  // dx/ds at (r_a, t_c)
+            }
+            // twice C_r = X_s x X_t
+            long long cr[3] = {geo_cross(xs[1], xt[2], xs[2], xt[1]) << 1, geo_cross(xs[2], xt[0], xs[0], xt[2]) << 1,
+                               geo_cross(xs[0], xt[1], xs[1], xt[0]) << 1};
+            const long long det = geo_dot<0>(xr, cr);  // |J| = det 2^(K3 - 59)
+            lost = lost || (det >> 32) < 1;
+            const int z = max(0, __clzll(det | 1) - 2);
+            const long long W = geo_mul<2>(w2, fw[c]);  // weights 2^(62 - kwc)
+            const int kwc = kw + (__double2hiint(sw[c]) >> 20) - 1022;
+            const long long dn = det << z;
+            const double wj = fx_to_double(geo_mul<2>(W, dn), kwc + K3 - 59 - z);
+            if (MIN) mindet = fmin(mindet, fx_to_double(det, K3 - 59));
+            if (kind == 1) {
+                ge[c * qq] = wj;
+            } else {
+                long long cs[3] = {geo_cross(xt[1], xr[2], xt[2], xr[1]) << 1, geo_cross(xt[2], xr[0], xt[0], xr[2]) << 1,
+                                   geo_cross(xt[0], xr[1], xt[1], xr[0]) << 1};
+                long long ct[3] = {geo_cross(xr[1], xs[2], xr[2], xs[1]) << 1, geo_cross(xr[2], xs[0], xr[0], xs[2]) << 1,
+                                   geo_cross(xr[0], xs[1], xr[1], xs[0]) << 1};
+                const long long f = geo_mul<3>(W, geo_recip(dn));  // W / |J| = f 2^(kwc - 64 - K3 + z)
+                const long long grr = geo_dot<2>(cr, cr), gss = geo_dot<2>(cs, cs), gtt = geo_dot<2>(ct, ct);
+                most |= (int)(grr >> 32) | (int)(gss >> 32) | (int)(gtt >> 32);
+                // G = (f g / 2^61) 2^(kwc - K3 + z + E_a + E_b + 59), E_r = ks + kt - 61, ...
+                const int k = kwc - K3 + z - 63;
                 double *g = ge + c * qq;
-                g[0 * QP] = f * (Cr0 * Cr0 + Cr1 * Cr1 + Cr2 * Cr2);
-                g[1 * QP] = f * (Cr0 * Cs0 + Cr1 * Cs1 + Cr2 * Cs2);
-                g[2 * QP] = f * (Cr0 * Ct0 + Cr1 * Ct1 + Cr2 * Ct2);
-                g[3 * QP] = f * (Cs0 * Cs0 + Cs1 * Cs1 + Cs2 * Cs2);
-                g[4 * QP] = f * (Cs0 * Ct0 + Cs1 * Ct1 + Cs2 * Ct2);
-                g[5 * QP] = f * (Ct0 * Ct0 + Ct1 * Ct1 + Ct2 * Ct2);
-                g[6 * QP] = W * det;
-                if (kind == 4) wj2[e * (int64_t)QP + c * qq + ab] = W * det;
+                g[0 * QP] = fx_to_double(geo_mul<3>(f, grr), k + 2 * (ks + kt));
+                g[1 * QP] = fx_to_double(geo_mul<3>(f, geo_dot<2>(cr, cs)), k + K3 + kt);
+                g[2 * QP] = fx_to_double(geo_mul<3>(f, geo_dot<2>(cr, ct)), k + K3 + ks);
+                g[3 * QP] = fx_to_double(geo_mul<3>(f, gss), k + 2 * (kr + kt));
+                g[4 * QP] = fx_to_double(geo_mul<3>(f, geo_dot<2>(cs, ct)), k + K3 + kr);
+                g[5 * QP] = fx_to_double(geo_mul<3>(f, gtt), k + 2 * (kr + ks));
+                g[6 * QP] = wj;
+                if (kind == 4) wj2[e * (int64_t)QP + c * qq + ab] = wj;
+            }
+        }
+        if (lost) scale[4] = 1;
+        if (most >= 1 << 30 || most < 0) scale[7] = 1;
+    }
+    __syncthreads();
+    const bool all = scale[4] | scale[5] | scale[6];
+    left = valid && (all || (kind != 1 && scale[7]));
+    if (__syncthreads_or(left)) {
+        // the same in FP64, for the elements that are left
+        if (left) {
+            // entry (u, v): X_r at (s_u, t_v), X_s at (r_u, t_v), X_t at (r_u, s_v)
+            const double p = sx[u], w2 = sx[v];
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                Xr[ab * 3 + d] = fma(w2, fma(p, K[(0 * 4 + 3) * 3 + d], K[(0 * 4 + 2) * 3 + d]),
+                                     fma(p, K[(0 * 4 + 1) * 3 + d], K[(0 * 4 + 0) * 3 + d]));
+                Xs[ab * 3 + d] = fma(w2, fma(p, K[(1 * 4 + 3) * 3 + d], K[(1 * 4 + 2) * 3 + d]),
+                                     fma(p, K[(1 * 4 + 1) * 3 + d], K[(1 * 4 + 0) * 3 + d]));
+                Xt[ab * 3 + d] = fma(w2, fma(p, K[(2 * 4 + 3) * 3 + d], K[(2 * 4 + 2) * 3 + d]),
+                                     fma(p, K[(2 * 4 + 1) * 3 + d], K[(2 * 4 + 0) * 3 + d]));
+            }
+        }
+        __syncthreads();
+        if (left) {
+            if (all) mindet = 1e300;
+            double xt[3];
+#pragma unroll
+            for (int d = 0; d < 3; d++) xt[d] = Xt[(a + qn * b) * 3 + d];  // dx/dt at (r_a, s_b)
+#pragma unroll 1
+            for (int c = 0; c < qn; c++) {
+                double xr[3], xs[3];
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    xr[d] = Xr[(b + qn * c) * 3 + d];  // dx/dr at (s_b, t_c)
+                    xs[d] = Xs[(a + qn * c) * 3 + d];  // dx/ds at (r_a, t_c)
+                }
+                // C_r = X_s x X_t
+                const double Cr0 = xs[1] * xt[2] - xs[2] * xt[1];
+                const double Cr1 = xs[2] * xt[0] - xs[0] * xt[2];
+                const double Cr2 = xs[0] * xt[1] - xs[1] * xt[0];
+                const double det = xr[0] * Cr0 + xr[1] * Cr1 + xr[2] * Cr2;
+                const double W = wab * sw[c];
+                if (MIN && all) mindet = fmin(mindet, det);
+                if (kind == 1) {
+                    ge[c * qq] = W * det;
+                } else {
+                    const double Cs0 = xt[1] * xr[2] - xt[2] * xr[1];
+                    const double Cs1 = xt[2] * xr[0] - xt[0] * xr[2];
+                    const double Cs2 = xt[0] * xr[1] - xt[1] * xr[0];
+                    const double Ct0 = xr[1] * xs[2] - xr[2] * xs[1];
+                    const double Ct1 = xr[2] * xs[0] - xr[0] * xs[2];
+                    const double Ct2 = xr[0] * xs[1] - xr[1] * xs[0];
+                    const double f = W * recip(det);
+                    {
+                        double *g = ge + c * qq;
+                        g[0 * QP] = f * (Cr0 * Cr0 + Cr1 * Cr1 + Cr2 * Cr2);
+                        g[1 * QP] = f * (Cr0 * Cs0 + Cr1 * Cs1 + Cr2 * Cs2);
+                        g[2 * QP] = f * (Cr0 * Ct0 + Cr1 * Ct1 + Cr2 * Ct2);
+                        g[3 * QP] = f * (Cs0 * Cs0 + Cs1 * Cs1 + Cs2 * Cs2);
+                        g[4 * QP] = f * (Cs0 * Ct0 + Cs1 * Ct1 + Cs2 * Ct2);
+                        g[5 * QP] = f * (Ct0 * Ct0 + Ct1 * Ct1 + Ct2 * Ct2);
+                        if (all) {
+                            g[6 * QP] = W * det;
+                            if (kind == 4) wj2[e * (int64_t)QP + c * qq + ab] = W * det;
+                        }
+                    }
+                }
             }
         }
     }
@@ -198,13 +370,12 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
     }
 }
 
-// Two resident blocks of about 512 threads per SM (a register cap of 64)
-// up to 10 points per direction, measured faster than the compiler's own
-// choice; above that the cap would spill.
-constexpr int geo_min_blocks(int qn) { return qn <= 10 ? 2 : 0; }
+// Resident blocks per SM that the register allocation must allow (64 and 80
+// registers; at 17 points 1068 us with three, 1195 with five).
+constexpr int geo_min_blocks(int qn) { return qn <= 10 ? 4 : 3; }
 
 template <int qn, int kind, bool MIN>
-__global__ void __launch_bounds__(GeoCfg<qn>::threads)
+__global__ void __launch_bounds__(GeoCfg<qn>::threads, geo_min_blocks(qn))
 geofacs_kernel(int64_t E, const double *__restrict__ nodes, const double *__restrict__ weights,
                const double *__restrict__ verts, double *__restrict__ geo, double *__restrict__ detJ_min,
                double *__restrict__ wj2) {
@@ -212,19 +383,8 @@ geofacs_kernel(int64_t E, const double *__restrict__ nodes, const double *__rest
 }
 
 template <int qn, int kind, bool MIN>
-__global__ void __launch_bounds__(GeoCfg<qn>::threads, geo_min_blocks(qn) > 0 ? geo_min_blocks(qn) : 1)
-geofacs_kernel_capped(int64_t E, const double *__restrict__ nodes, const double *__restrict__ weights,
-                      const double *__restrict__ verts, double *__restrict__ geo, double *__restrict__ detJ_min,
-                      double *__restrict__ wj2) {
-    geofacs_body<qn, kind, MIN>(E, nodes, weights, verts, geo, detJ_min, wj2);
-}
-
-template <int qn, int kind, bool MIN>
 constexpr auto geo_fn() {
-    if constexpr (geo_min_blocks(qn) > 0)
-        return &geofacs_kernel_capped<qn, kind, MIN>;
-    else
-        return &geofacs_kernel<qn, kind, MIN>;
+    return &geofacs_kernel<qn, kind, MIN>;
 }
 
 template <int N>

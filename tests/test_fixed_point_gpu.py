@@ -208,3 +208,44 @@ def test_element_counts_around_the_blocks(name, N):
     full = _check(op, geo, q)
     for E in (1, 2, 3, 7, 31, 32, 33):
         np.testing.assert_array_equal(op.apply(geo[:E], q[:E]), full[:E])
+
+
+def _hexahedra():
+    """An ordinary element, a box, a sheared, a rotated and a strongly
+    distorted one, one with a skew of 1e-5, a flat, a large, a tiny and an
+    inverted one."""
+    rng = np.random.default_rng(3)
+    box = np.array([[(c >> d) & 1 for d in range(3)] for c in range(8)], dtype=float)
+    jitter = rng.uniform(-1, 1, (8, 3))
+    rot = np.linalg.qr(rng.standard_normal((3, 3)))[0]
+    rot *= np.sign(np.linalg.det(rot))
+    shear = np.array([[1, 0.7, -0.4], [0, 1, 0.8], [0, 0, 1.0]])
+    v = [box + 0.1 * jitter, box, box @ shear.T, (box + 0.05 * jitter) @ rot.T, box + 0.2 * jitter,
+         box + 1e-5 * jitter, box * [1, 1, 1e-3] + 1e-5 * jitter, 2.0 ** 90 * (box + 0.1 * jitter),
+         2.0 ** -90 * (box + 0.1 * jitter), (box + 0.1 * jitter)[[1, 0, 3, 2, 5, 4, 7, 6]]]
+    return np.ascontiguousarray(np.array(v))
+
+
+@pytest.mark.parametrize("N", [1, 2, 4, 7, 8, 9, 15])
+def test_factors_of_elements_of_every_kind(N):
+    """Geometric factors, fixed-point or FP64 by element: each within 1e-13 of
+    the oracle relative to sqrt(Gaa Gbb) (about 40 roundings at a cancellation
+    of up to 20 in the determinant) times the ratio of the element's largest
+    coordinate to its shortest edge (the columns of the map are differences of
+    coordinates, which the oracle rounds at the coordinates' size), wJ the same
+    bits from every entry point, and the same bits for an element alone."""
+    fem = _fem()
+    b, verts = fem.fem_basis_setup(N), _hexahedra()
+    edges = np.stack([verts[:, i] - verts[:, j] for i, j in ((1, 0), (2, 0), (4, 0), (7, 6), (7, 5), (7, 3))], 1)
+    ratio = np.abs(verts).max((1, 2)) / np.linalg.norm(edges, axis=2).min(1)
+    for kind in (fem.FEM_GEO_BP35, fem.FEM_GEO_BP30):
+        got = fem.fem_mesh_geofacs(b, kind, _dev(verts)).cpu().numpy()
+        ref = oracle.geofacs(N, kind, verts)[0]
+        d = np.sqrt(np.abs(ref[:, [0, 3, 5]]))
+        scale = np.stack([d[:, 0] ** 2, d[:, 0] * d[:, 1], d[:, 0] * d[:, 2], d[:, 1] ** 2, d[:, 1] * d[:, 2],
+                          d[:, 2] ** 2, np.abs(ref[:, 6])], 1)
+        assert np.all(np.abs(got - ref) <= 1e-13 * ratio[:, None, None] * scale)
+        for e in (1, 5, 9):
+            np.testing.assert_array_equal(fem.fem_mesh_geofacs(b, kind, _dev(verts[e:e + 1])).cpu().numpy()[0], got[e])
+    wj = fem.fem_mesh_geofacs(b, fem.FEM_GEO_BP1, _dev(verts)).cpu().numpy()
+    np.testing.assert_array_equal(wj, got[:, 6])
