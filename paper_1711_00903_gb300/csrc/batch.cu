@@ -181,7 +181,7 @@ batch_kernel(const BatchMesh *__restrict__ meshes, const BatchTask *__restrict__
 
 FEM_DEFINE_FX_UPLOAD(upload_fold_batch_tu)
 
-// FP64 instructions per element (even-odd lines; used to order tasks).
+// Multiply-adds per element of the even-odd lines, used to order tasks.
 double cost_per_element(int op, int N) {
     const int n = N + 1, m = N + 2;
     return op == FEM_OP_BP30 ? (double)m * m * m * (2.0 * m + 30) + 4.0 * n * n * n * m

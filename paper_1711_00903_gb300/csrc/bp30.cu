@@ -1,11 +1,12 @@
-// BP3.0 dealiased screened-Poisson matvec, IEEE FP64 (Algorithm 5):
+// BP3.0 dealiased screened-Poisson matvec in FP32 (Algorithm 5; the FP64
+// operator is in bp30_fx.cu):
 //   Aq = (I^T x I^T x I^T) [ Dt_r^T Rr + Dt_s^T Rs + Dt_t^T Rt + lambda wJ qg ],
 //   qg = (I x I x I) q,  [Rr Rs Rt] = G [Dt_r qg, Dt_s qg, Dt_t qg],
 // twelve one-dimensional contractions per element in one kernel with no
 // global intermediates (Section 8: a three-kernel split was no faster, and
 // removing global intermediates was the largest gain).
 //
-// GB300 design.  Bound by FP64 instruction issue (2 per clock per SM), so
+// GB300 design.  Bound by instruction issue and the factors' traffic, so
 // every contraction is one thread applying an even-odd folded operator to
 // a whole line with constant-bank operands (eo.cuh), and the element lives
 // in three m^3 shared-memory boxes:
@@ -45,7 +46,7 @@ bp30_kernel(int64_t E, const T *__restrict__ G, double lambda, const T *__restri
 }
 
 template <typename T, int N, bool PCG>
-__global__ void __launch_bounds__(Bp30Cfg<N, T>::threads, bp30_min_blocks<T, N>())
+__global__ void __launch_bounds__(Bp30Cfg<N, T>::threads, bp30_min_blocks<N>())
 bp30_kernel_capped(int64_t E, const T *__restrict__ G, double lambda, const T *__restrict__ q, T *__restrict__ Aq,
                    const T *__restrict__ z, T *__restrict__ p, const double *__restrict__ beta,
                    double *__restrict__ partials) {
@@ -54,7 +55,7 @@ bp30_kernel_capped(int64_t E, const T *__restrict__ G, double lambda, const T *_
 
 template <typename T, int N, bool PCG>
 constexpr auto bp30_fn() {
-    if constexpr (bp30_min_blocks<T, N>() > 0)
+    if constexpr (bp30_min_blocks<N>() > 0)
         return &bp30_kernel_capped<T, N, PCG>;
     else
         return &bp30_kernel<T, N, PCG>;
@@ -71,10 +72,8 @@ struct Bp30LaunchT {
         static cudaError_t run(int64_t E, const T *G, double lambda, const T *q, T *Aq, const T *z, T *p,
                                const double *beta, double *partials, cudaStream_t s, double *status = nullptr,
                                int which = 0) {
-            if constexpr (sizeof(T) == 4) {
-                if (which == 2 || (which == 0 && bp30_stream_default(N, false, PCG)))
-                    return launch_bp30_stream(N, PCG, E, G, lambda, q, Aq, z, p, beta, partials, s, status);
-            }
+            if (which == 2 || (which == 0 && bp30_stream_default(N, false, PCG)))
+                return launch_bp30_stream(N, PCG, E, G, lambda, q, Aq, z, p, beta, partials, s, status);
             using C = Bp30Cfg<N, T>;
             const int64_t blocks = (E + C::EPB - 1) / C::EPB;
             bp30_fn<T, N, PCG>()<<<(unsigned)blocks, C::threads, C::smem, s>>>(E, G, lambda, q, Aq, z, p, beta,

@@ -27,7 +27,7 @@ __device__ __forceinline__ void f16g30_entry(int64_t E, const __half *__restrict
 // than the FP32 cap of four; the FP32 operator itself lost 6 % with six.
 template <int N>
 constexpr int bp30_f16_min_blocks() {
-    return N == 9 ? 6 : bp30_min_blocks<float, N>();
+    return N == 9 ? 6 : bp30_min_blocks<N>();
 }
 
 template <int N, bool PCG>

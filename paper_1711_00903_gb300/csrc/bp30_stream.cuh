@@ -154,8 +154,8 @@ bp30_stream_kernel(int64_t E, const TG *__restrict__ G, double lambda, const flo
         __syncthreads();
 
         const Hooks hooks{&bar[0], (unsigned)(it & 1), &failed, &pend_g, has_next, g + gridDim.x, &issue_g};
-        dot += (double)bp30_core<N, EPS, float, PCG, true, TG, false, Hooks>(boxes, e0, nel, sG, lambda, Aq, p,
-                                                                             gscale, nullptr, hooks);
+        dot += (double)bp30_core<N, EPS, float, PCG, true, TG, Hooks>(boxes, e0, nel, sG, lambda, Aq, p,
+                                                                             gscale, hooks);
         if (failed) break;
         __syncthreads();  // the boxes and the field stage are free again
     }

@@ -47,8 +47,7 @@ struct Bp35Layout {
     };
     // FP32 is bound by HBM: at kernel start one thread asks the TMA engine
     // to prefetch the block's factor planes (one contiguous range) into L2,
-    // so that the chain-rule phase finds them there.  FP64 is bound by FP64
-    // issue and reads the factors directly.
+    // so that the chain-rule phase finds them there.
     static constexpr bool PREFETCH = sizeof(T) == 4;
     static constexpr int EPB = EPB_;
     static constexpr int threads = ((nn * EPB + 31) / 32) * 32;  // the block needs at least this many
@@ -213,8 +212,8 @@ __device__ __forceinline__ void bp35_block(unsigned char *smem_raw, int64_t e0, 
 // Minimum resident blocks per SM that the register allocation must allow
 // (0: the compiler's own heuristic).  At high degree the fully unrolled line
 // kernels take up to 255 registers and leave one block per SM; capping them
-// trades a few spills for latency hiding.  Chosen per precision and degree
-// from the operator sweep on GB300.
+// trades a few spills for latency hiding.  Chosen per degree from the operator
+// sweep on GB300.
 template <typename T, int N>
 constexpr int bp35_min_blocks() {
     return N == 15 ? 3 : 0;

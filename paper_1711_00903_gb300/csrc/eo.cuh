@@ -10,9 +10,8 @@
 // and a middle output row (P odd) uses e (sigma = +1) or o (sigma = -1)
 // only (Solomonoff 1992; Kopriva, "Implementing Spectral Methods for PDEs",
 // 2009).  A line of Q inputs and P outputs then costs about P Q / 2 FMAs
-// plus P + Q adds instead of P Q FMAs.  On GB300, where FP64 issues at
-// 2 instructions per clock per SM, that is the quantity that bounds the
-// FP64 operators.
+// plus P + Q adds instead of P Q FMAs.  The FP32 lines are here; the FP64
+// operators apply the same folded lines in 64-bit fixed point (fx.cuh).
 //
 // The folded matrices of every degree live in one __constant__ table; each
 // kernel reads them at compile-time offsets, so every operator entry is a
@@ -38,24 +37,22 @@ namespace fem {
 
 // ------------------------------------------------------------ device side
 
-// One constant table per translation unit and precision (no relocatable
-// device code); every TU that uses them uploads the same contents at basis
-// setup.
+// One constant table per translation unit (no relocatable device code); every
+// TU that uses it uploads the same contents at basis setup.
 //
-// Translation units whose constant bank holds the fixed-point tables of
-// fx.cuh (FEM_FX_TABLES) keep this FP64 table in global memory: their FP64
-// lines are the exception there, and a load per FMA hides behind the FP64
-// pipe (2 per clock per SM).
+// Translation units of the fixed-point operators (FEM_FX_TABLES) hold the FP64
+// table instead, in global memory (their constant bank holds the fixed-point
+// tables of fx.cuh): FP64 lines are the exception there, and a load per FMA
+// hides behind the FP64 pipe (2 per clock per SM).
 #ifdef FEM_FX_TABLES
 static __device__ double c_fold[kFoldTotal];
-#else
-static __constant__ double c_fold[kFoldTotal];
 #endif
 static __constant__ float2 c_fold32p[kFoldPairTotal];
 
-// FP32 form of eo_apply below (the pair table, OFF its folded offset).
+// y (P) = A x (Q) along one line in FP32, A folded at table offset OFF, parity
+// SIG.
 template <int P, int Q, int SIG, int OFF>
-__device__ __forceinline__ void eo_apply_f32(const float (&x)[Q], float (&y)[P]) {
+__device__ __forceinline__ void eo_apply(const float (&x)[Q], float (&y)[P]) {
     constexpr int hp = P / 2, hq = Q / 2;
     constexpr int oP = fold_pair_offset_of(OFF);
     static_assert(oP >= 0, "no folded operator block starts at this offset");
@@ -81,51 +78,6 @@ __device__ __forceinline__ void eo_apply_f32(const float (&x)[Q], float (&y)[P])
         if ((Q % 2) && SIG > 0) M = fmaf(c_fold32p[oR + hq].x, x[hq], M);
         y[hp] = M;
     }
-}
-
-
-// FP64 form of eo_apply below.
-template <int P, int Q, int SIG, int OFF, typename T>
-__device__ __forceinline__ void eo_apply_f64(const T (&x)[Q], T (&y)[P]) {
-    constexpr int hp = P / 2, hq = Q / 2;
-    constexpr int oS = OFF, oT = OFF + hp * hq, oC = OFF + 2 * hp * hq;
-    constexpr int oR = oC + ((Q % 2) ? hp : 0);
-    T e[hq > 0 ? hq : 1], o[hq > 0 ? hq : 1];
-#pragma unroll
-    for (int i = 0; i < hq; i++) {
-        e[i] = x[i] + x[Q - 1 - i];
-        o[i] = x[i] - x[Q - 1 - i];
-    }
-#pragma unroll
-    for (int a = 0; a < hp; a++) {
-        T E = T(0), O = T(0);
-#pragma unroll
-        for (int i = 0; i < hq; i++) {
-            E = fmx(c_fold[oS + a * hq + i], e[i], E);
-            O = fmx(c_fold[oT + a * hq + i], o[i], O);
-        }
-        if (Q % 2) E = fmx(c_fold[oC + a], x[hq], E);
-        y[a] = E + O;
-        y[P - 1 - a] = (SIG > 0) ? (E - O) : (O - E);
-    }
-    if (P % 2) {
-        T M = T(0);
-#pragma unroll
-        for (int i = 0; i < hq; i++) M = fmx(c_fold[oR + i], (SIG > 0) ? e[i] : o[i], M);
-        if ((Q % 2) && SIG > 0) M = fmx(c_fold[oR + hq], x[hq], M);
-        y[hp] = M;
-    }
-}
-
-// y (P) = A x (Q) along one line, A folded at table offset OFF, parity SIG,
-// in the precision T of the data.
-template <int P, int Q, int SIG, int OFF, typename T>
-__device__ __forceinline__ void eo_apply(const T (&x)[Q], T (&y)[P]) {
-    static_assert(std::is_same<T, float>::value || std::is_same<T, double>::value, "FP32 or FP64 lines");
-    if constexpr (std::is_same<T, float>::value)
-        eo_apply_f32<P, Q, SIG, OFF>(x, y);
-    else
-        eo_apply_f64<P, Q, SIG, OFF>(x, y);
 }
 
 // Padded element box q1 x q2 x q3 (i fastest); an odd row stride keeps the
@@ -222,8 +174,8 @@ __device__ __forceinline__ void for_tasks(int nel, F &&f) {
     }
 }
 
-// Host: uploads the folded table (kFoldTotal doubles) to this TU's copies:
-// the FP64 table as it is, the FP32 pair table rounded from it.
+// Host: rounds the folded table (kFoldTotal doubles) to this TU's FP32 pair
+// table.
 #define FEM_DEFINE_FOLD_UPLOAD(NAME)                                                      \
     cudaError_t NAME(const double *table) {                                               \
         static float2 tp[kFoldPairTotal];                                                 \
@@ -236,9 +188,6 @@ __device__ __forceinline__ void for_tasks(int nel, F &&f) {
                 for (int k = 0; k < hh; k++) o[k] = make_float2((float)f[k], (float)f[hh + k]); \
                 for (int k = 0; k < rest; k++) o[hh + k] = make_float2((float)f[2 * hh + k], 0.0f); \
             }                                                                             \
-        cudaError_t e = cudaMemcpyToSymbol(c_fold, table, sizeof(double) * kFoldTotal, 0,  \
-                                           cudaMemcpyHostToDevice);                       \
-        if (e != cudaSuccess) return e;                                                   \
         return cudaMemcpyToSymbol(c_fold32p, tp, sizeof(float2) * kFoldPairTotal, 0,     \
                                   cudaMemcpyHostToDevice);                                \
     }

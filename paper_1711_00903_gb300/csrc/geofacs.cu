@@ -50,8 +50,8 @@ struct GeoCfg {
 // the full 53).  The seed's conversions between the IEEE binary64 and
 // binary32 formats are done on the bit fields with integer operations
 // (sign; exponent rebiased from 1023 to 127; the top 23 mantissa bits,
-// truncated), so the FP64 pipe, the part's bottleneck, executes only the
-// four FMAs.  Falls back to a division when |d| is outside 2^-120..2^121,
+// truncated), so the FP64 pipe (2 per clock per SM) executes only the four
+// FMAs.  Falls back to a division when |d| is outside 2^-120..2^121,
 // where the seed or its reciprocal would leave the binary32 normal range.
 __device__ __forceinline__ double recip(double d) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(d);
