@@ -47,9 +47,9 @@ KERNELS = ["geofacs_bp35", "geofacs_bp30_bp1", "bp35", "bp1_bp30"]
 # a kernel whose source changed since reports traffic null.
 NCU_TRAFFIC = {
     # ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch on E = 4096:
-    # (184.09 + 19.69) MB over 4096 elements, ncu capture of the one-pass kernel at N = 7
-    "bp1_bp30": {"N": 7, "bytes_per_elem": 49750, "sha": "63b3cce49d1ad5cd",
-                 "files": ["bp30.cu", "bp30_body.cuh", "eo.cuh", "kernels_common.cuh"]},
+    # (185.61 + 24.01) MB over 4096 elements, ncu capture of the one-pass kernel at N = 7
+    "bp1_bp30": {"N": 7, "bytes_per_elem": 51176, "sha": "e943693162630f1c",
+                 "files": ["bp30_fx.cu", "bp30_fx.cuh", "fx.cuh", "fx_point.cuh"]},
 }
 
 
@@ -73,13 +73,42 @@ def fp64_peak_tflops(sm_mhz: float) -> float:
     return SMS * FP64_INST_PER_CLK_SM * 2 * sm_mhz * 1e6 / 1e12
 
 
+# 32 x 32 + 64-bit integer multiply-adds, the instruction of the FP64 operators'
+# fixed-point contractions: 29 per clock per SM measured with independent
+# chains of mad.lo.cc + madc.hi (one instruction)
+IMAD_PER_CLK_SM = 29
+
+
+def imad_peak_ginst(sm_mhz: float) -> float:
+    return SMS * IMAD_PER_CLK_SM * sm_mhz * 1e6 / 1e9
+
+
+def imad_counts(N: int):
+    """Integer multiply-adds per element of the fixed-point kernels: three per
+    folded multiply-add of a contraction and per product of the chain rule (9
+    and the mass term) or of BP1.0's wJ q, about 150 per point of the factors."""
+    n, m = N + 1, N + 2
+    n3, m3, mm, nn = n ** 3, m ** 3, m * m, n * n
+    fma = {k: f - i for k, (i, f) in (("mn", eo_cost(m, n, 1)), ("nm", eo_cost(n, m, 1)), ("dd", eo_cost(n, n, -1)),
+                                      ("gg", eo_cost(m, m, -1)))}
+    lines = nn + m * n + mm
+    return {
+        "bp1": 3 * (lines * (fma["mn"] + fma["nm"]) + m3),
+        "bp35": 3 * (6 * nn * fma["dd"] + 10 * n3),
+        "bp30": 3 * (lines * (fma["mn"] + fma["nm"]) + 6 * mm * fma["gg"] + 10 * m3),
+        "bp1_bp30": 3 * (lines * (fma["mn"] + 2 * fma["nm"]) + 6 * mm * fma["gg"] + 11 * m3),
+        "geofacs_bp30_bp1": 150 * m3,
+        "geofacs_bp35": 150 * n3,
+    }
+
+
 def fp64_peak_ginst(sm_mhz: float) -> float:
     return SMS * FP64_INST_PER_CLK_SM * sm_mhz * 1e6 / 1e9
 
 
 def eo_cost(P: int, Q: int, sig: int):
-    """(FP64 instructions, flops) of one even-odd folded line y(P) = A x(Q)
-    as the kernels execute it: Q/2 fold pairs (2 adds each), per output pair
+    """(instructions, flops) of one even-odd folded line y(P) = A x(Q) in
+    floating point: Q/2 fold pairs (2 adds each), per output pair
     2(Q/2) + Q%2 FMAs and 2 adds, a middle output row of Q/2 (+1) FMAs."""
     hp, hq = P // 2, Q // 2
     fma = hp * (2 * hq + Q % 2) + (P % 2) * (hq + (1 if (Q % 2 and sig > 0) else 0))
@@ -93,7 +122,9 @@ def alg_counts(N: int):
              multiply-add = 2 flops): BP1.0 4(mn^3+m^2n^2+m^3n)+m^3, BP3.5
              12n^4+18n^3, BP3.0 4(mn^3+m^2n^2+m^3n)+12m^4+18m^3; for the
              geometric factors the flops the kernel executes;
-    inst  -- FP64 instructions the kernels execute (even-odd lines);
+    inst  -- FP64 instructions of the even-odd lines in floating point: what
+             the point layouts execute, and what the fixed-point kernels
+             would have to issue on the FP64 pipe instead;
     bytes -- algorithmic HBM bytes (Table 1 of the paper for the operators;
              24 vertex doubles in and the planes out for the factors)."""
     n, m = N + 1, N + 2
@@ -541,6 +572,7 @@ def run_ours(args):
     value = world * dofs * args.steps / (ms / 1e3) / 1e9
     std, inst, byts = alg_counts(N)
     smem = smem_counts(N)
+    imad = imad_counts(N)
     hbm, hbm_src, _ = _peaks()
     sm_mhz = clocks.get("sm_mhz") or 2070.0
     kern = {}
@@ -555,13 +587,13 @@ def run_ours(args):
             "fp64_tflops": E * std[name] / t / 1e12,
             "fp64_frac": E * std[name] / t / 1e12 / fp64_peak_tflops(2070.0),
             "fp64_issue_frac": E * inst[name] / t / 1e9 / fp64_peak_ginst(sm_mhz),
+            "imad_frac": E * imad[name] / t / 1e9 / imad_peak_ginst(sm_mhz),
             "smem_frac": E * smem[name] / t / 1e9 / smem_peak_gbs(sm_mhz) if name in smem else None,
         }
     dom = max(KERNELS, key=lambda k: per_kernel[k])
     tr = NCU_TRAFFIC.get(dom)
     traffic = tr["bytes_per_elem"] * E if tr and tr["sha"] == _src_hash(tr["files"]) and tr["N"] == N else None
-    peak_alu = fp64_peak_tflops(2070.0)
-    # the FP64 ceiling measured on this GPU: independent FMA chains on every SM
+    # the FP64 rate measured on this GPU: independent FMA chains on every SM
     probe_out, probe_flops = fem.fem_fma_probe(10000)
     fem.fem_fma_probe(10000, out=probe_out)
     pe0, pe1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -573,17 +605,15 @@ def run_ours(args):
     probe_tflops = 3 * probe_flops / (pe0.elapsed_time(pe1) / 1e3) / 1e12
     del probe_out
     roofline = {
-        "kernel": dom, "bound": "alu", "unit": "TFLOP/s",
-        "achieved": kern[dom]["fp64_tflops"], "peak": peak_alu,
-        "frac": kern[dom]["fp64_tflops"] / peak_alu,
-        "peak_source": "FP64 issue rate derived from unit counts: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2070 MHz",
-        "flop_count": "direct sum factorisation (multiply-add = 2); the even-odd folded kernels execute "
-                      "about 0.65x of these at N=7, so frac can exceed 1",
+        "kernel": dom, "bound": "alu", "unit": "Gimad/s",
+        "achieved": E * imad[dom] / (per_kernel[dom] / 1e3) / 1e9, "peak": imad_peak_ginst(sm_mhz),
+        "frac": kern[dom]["imad_frac"],
+        "peak_source": "32x32+64-bit integer multiply-adds: 152 SMs x 29/clk measured x median SM clock",
+        "flop_count": "3 integer multiply-adds per even-odd folded multiply-add and chain-rule product",
+        # the folded lines' floating-point instructions over the FP64 pipe's
+        # rate: above 1 the fixed-point kernel runs faster than that pipe could
         "fp64_issue_frac": kern[dom]["fp64_issue_frac"],
         "fp64_probe_tflops": probe_tflops,
-        # FP64 instructions per second of the kernel over those of the probe
-        # (2 flops per probe instruction): the fraction of the FP64 rate this
-        # GPU sustains
         "fp64_issue_frac_of_probe": kern[dom]["fp64_issue_frac"] * fp64_peak_ginst(sm_mhz) / (probe_tflops * 1e3 / 2),
         "fp64_probe": "measured FP64 FMA rate of this GPU (fem_fma_probe: 8 independent FMA chains per thread, "
                       "8 x 256 threads per SM)",

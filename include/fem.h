@@ -123,9 +123,16 @@ int fem_mesh_geofacs(const fem_basis *b, fem_geo_kind kind, int64_t E,
 int fem_mesh_geofacs_set(const fem_basis *b, int64_t E, const double *verts, double *wJ,
                          double *G35, double *G30, void *stream);
 
+/* Arithmetic of the FP64 operators and factors below: FP64 in and out; inside,
+ * 64-bit fixed point scaled per element (60-61 bits, more than FP64's 53), with
+ * IEEE FP64 for every element whose values do not share a scale (a range wider
+ * than the fixed point holds, infinities, NaN).  The error against exact
+ * arithmetic is at most that of the same lines in IEEE FP64; an element's
+ * result depends on that element alone. */
+
 /* BP1.0 mass matvec (Algorithm 3: interpolate GLL -> Gauss with
  * I x I x I (Algorithm 1), scale by wJ, project with I^T x I^T x I^T
- * (Algorithm 2)), six tensor contractions per element, IEEE FP64.
+ * (Algorithm 2)), six tensor contractions per element.
  *   wJ device E*NpG, q device E*Np, Mq device E*Np (must not overlap q, wJ).
  * E == 0 enqueues nothing.  Errors: FEM_EINVAL, FEM_ECUDA. */
 int fem_bp1_apply(const fem_basis *b, int64_t E, const double *wJ, const double *q,
@@ -134,7 +141,7 @@ int fem_bp1_apply(const fem_basis *b, int64_t E, const double *wJ, const double 
 /* BP3.5 collocated screened-Poisson matvec (Algorithm 4): derivatives
  * along r, s, t with D, the symmetric chain rule with the six G factors,
  * D^T along each direction, plus lambda * wJ * q at the GLL nodes; six
- * tensor contractions per element, IEEE FP64.
+ * tensor contractions per element.
  *   G device E*7*Np, q device E*Np, Aq device E*Np (must not overlap q, G).
  * E == 0 enqueues nothing.  Errors: FEM_EINVAL, FEM_ECUDA. */
 int fem_bp35_apply(const fem_basis *b, int64_t E, const double *G, double lambda,
@@ -143,7 +150,7 @@ int fem_bp35_apply(const fem_basis *b, int64_t E, const double *G, double lambda
 /* BP3.0 dealiased screened-Poisson matvec (Algorithm 5): interpolate to
  * the Gauss points, differentiate there with Dt, apply the chain rule with
  * G, apply Dt^T, add lambda * wJ times the interpolated field, project
- * with I^T; twelve tensor contractions per element, IEEE FP64.
+ * with I^T; twelve tensor contractions per element.
  *   G device E*7*NpG, q device E*Np, Aq device E*Np (must not overlap q, G).
  * E == 0 enqueues nothing.  Errors: FEM_EINVAL, FEM_ECUDA. */
 int fem_bp30_apply(const fem_basis *b, int64_t E, const double *G, double lambda,
@@ -155,8 +162,8 @@ int fem_bp30_apply(const fem_basis *b, int64_t E, const double *G, double lambda
 int fem_bp35_apply_f32(const fem_basis *b, int64_t E, const float *G, double lambda,
                        const float *q, float *Aq, void *stream);
 
-/* FP64 issue-rate probe (the FP64 ceiling of the operators is measured, not
- * assumed): fem_fma_probe_threads() threads (8 blocks of 256 per SM of the
+/* FP64 issue-rate probe (the rate of the point layouts and of the elements
+ * that stay in FP64 is measured, not assumed): fem_fma_probe_threads() threads (8 blocks of 256 per SM of the
  * current device) each run eight independent FP64 FMA chains of iters steps
  * and store one double to out (device, fem_fma_probe_threads() doubles).
  * One launch performs 2 * 8 * iters * threads flops; time it on stream.
