@@ -1,0 +1,104 @@
+"""Where 64-bit fixed point, scaled per element, would hold fewer digits than
+FP64 arithmetic: elements with nearly parallel edges (geometric factors) and
+flat elements (operators).  Against references in extended precision
+(np.longdouble: 64 bits of mantissa or more)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+LD = np.longdouble
+U = 2.0 ** -53
+BOX = np.array([[(c >> d) & 1 for d in range(3)] for c in range(8)], dtype=float)
+PAIRS = ((0, 0), (0, 1), (0, 2), (1, 1), (1, 2), (2, 2))
+
+
+def _fem():
+    import paper_1711_00903_gb300 as fem
+    return fem
+
+
+def _dev(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).to("cuda")
+
+
+def _rotation(rng):
+    r = np.linalg.qr(rng.standard_normal((3, 3)))[0]
+    return r * np.sign(np.linalg.det(r))
+
+
+def _columns(cols):
+    """The parallelepiped with these edge vectors, right-handed."""
+    cols = np.asarray(cols)
+    return BOX @ (cols if np.linalg.det(cols) > 0 else cols[[1, 0, 2]])
+
+
+def _parallel_elements():
+    """Rotated boxes sheared by 10 to 1e5, columns (1, +-a, +-a), two columns
+    that differ by 1e-3 to 1e-7, rotated flat elements."""
+    rng = np.random.default_rng(17)
+    v = []
+    for s in (3, 10, 100, 1e3, 1e4, 1e5):
+        for _ in range(3):
+            v.append(BOX @ np.array([[1, s, 0], [0, 1, 0], [0, 0, 1.0]]).T @ _rotation(rng).T)
+    for a in (0.3, 0.1, 0.04, 0.02, 0.012):
+        for _ in range(4):
+            v.append(_columns([[1, *(rng.choice([-1, 1], 2) * a * rng.uniform(0.7, 1.3, 2))] for _ in range(3)]))
+    for e in (1e-3, 1e-6, 1e-7):
+        for _ in range(3):
+            c = rng.uniform(0.5, 1, 3)
+            v.append(_columns([c, c + e * rng.uniform(-1, 1, 3), rng.uniform(-1, 1, 3)]))
+    for a in (10, 1e3):
+        v.append((BOX + 0.1 * rng.uniform(-1, 1, (8, 3))) * [1, 1, 1 / a] @ _rotation(rng).T)
+    return np.ascontiguousarray(np.array(v))
+
+
+def _factors(verts, x, w):
+    """Factors and, with u = 2^-53, the first-order bound of an evaluation in
+    FP64: 8 u per column component (edge differences and bilinear form, on
+    absolute values), 2 u per product of a cofactor, 6 u for the determinant,
+    the quotient and the weights, 4 u for the sum of three products."""
+    x, w = x.astype(LD), w.astype(LD)
+    h, d = np.stack([(1 - x) / 2, (1 + x) / 2], -1), np.stack([0 * x - 0.5, 0 * x + 0.5], -1)
+    v = verts.astype(LD).reshape(-1, 2, 2, 2, 3)
+
+    def columns(v, d):
+        return [np.einsum("etsrd,kt,js,ir->ekjid", v, *m) for m in ((h, h, d), (h, d, h), (d, h, h))]
+
+    X = columns(v, d)
+    e = [np.abs(np.diff(v, axis=a)).sum((1, 2, 3)) for a in (3, 2, 1)]  # |edges| along r, s, t
+    A = [0.5 * a[:, None, None, None, :] + 0 * X[0] for a in e]         # of the columns' components
+    cross = lambda a, b: np.stack([a[..., 1] * b[..., 2] + a[..., 2] * b[..., 1],  # noqa: E731
+                                   a[..., 2] * b[..., 0] + a[..., 0] * b[..., 2],
+                                   a[..., 0] * b[..., 1] + a[..., 1] * b[..., 0]], -1)
+    nxt = ((1, 2), (2, 0), (0, 1))
+    C = [np.cross(X[i], X[j]) for i, j in nxt]
+    dC = [U * (8 * (cross(A[i], abs(X[j])) + cross(abs(X[i]), A[j])) + 2 * cross(abs(X[i]), abs(X[j]))) for i, j in nxt]
+    det = (X[0] * C[0]).sum(-1)
+    ddet = (abs(X[0]) * dC[0] + 8 * U * A[0] * abs(C[0]) + 4 * U * abs(X[0] * C[0])).sum(-1)
+    W = w[:, None, None] * w[:, None] * w
+    G, bar = [], []
+    for a, b in PAIRS:
+        g = (C[a] * C[b]).sum(-1) * W / det
+        G.append(g)
+        bar.append(W / abs(det) * (dC[a] * abs(C[b]) + abs(C[a]) * dC[b] + 4 * U * abs(C[a] * C[b])).sum(-1)
+                   + abs(g) * (ddet / abs(det) + 6 * U))
+    G.append(W * det)
+    bar.append(W * ddet + 6 * U * abs(G[-1]))
+    shape = (verts.shape[0], 7, -1)
+    return np.stack(G, 1).reshape(shape), np.stack(bar, 1).reshape(shape)
+
+
+@pytest.mark.parametrize("N", [1, 2, 7, 15])
+def test_factors_of_nearly_parallel_edges(N):
+    """Each factor within the error that an evaluation in FP64 may have."""
+    fem = _fem()
+    b, verts = fem.fem_basis_setup(N), _parallel_elements()
+    t = fem.fem_basis_host_tables(N)
+    for kind, x, w in ((fem.FEM_GEO_BP35, "r", "w"), (fem.FEM_GEO_BP30, "rt", "wt")):
+        got = fem.fem_mesh_geofacs(b, kind, _dev(verts)).cpu().numpy()
+        ref, bar = _factors(verts, t[x], t[w])
+        assert np.all(abs(got - ref) <= bar)
+    wj = fem.fem_mesh_geofacs(b, fem.FEM_GEO_BP1, _dev(verts)).cpu().numpy()
+    np.testing.assert_array_equal(wj, got[:, 6])
