@@ -12,7 +12,8 @@
 //      line's (three in a row at the worst case's scale would lose 6 to 9
 //      bits);
 //   3. BP3.0: derivatives, scaled up by their largest value; chain rule with
-//      the factors scaled to 62 bits; transposes, each line scaled up by its
+//      the factors scaled to 62 bits (on flat elements direction by direction,
+//      FxScales); transposes, each line scaled up by its
 //      largest value; their sum with lambda wJ q, aligned, scaled up by its
 //      largest value; the three projections.
 // BP1.0 computed beside BP3.0 takes the same steps on the same numbers as
@@ -22,8 +23,8 @@
 // its values are not finite or extreme, when one of its eight octants holds
 // no value near its largest (the FP64 result there would keep digits that
 // the element's scale cuts off), when a point's factors are far below the
-// element's largest, or when the factors are not positive definite; element
-// by element, so a result does not depend on the block's other elements.
+// element's largest, when the factors are not positive definite or, at N = 1,
+// when the lines hold far less than their directions' scale; element by element, so a result does not depend on the block's other elements.
 //
 // What bounds it: integer multiply-adds and, between barriers, latency; see
 // bp30_fx.cu and bp1_fx.cu for the measured rates.
@@ -43,11 +44,15 @@ namespace {
 __host__ __device__ constexpr int fx30_octant_range(int N) { return N == 1 ? 2047 : kFxRange; }
 
 // Slots of an element's statistics: the eight octants of q, the largest wJ,
-// Grr, Gss, Gtt, derivative and sum at the Gauss points, whether the element
-// is left to FP64 (BP1.0, BP3.0), the largest value after the projection along
-// t (BP1.0, BP3.0) and after the interpolation along s, and the largest scale
-// of a transposed line (as 63 - its scale-up).
-enum { kFxW = 8, kFxG = 9, kFxU = 12, kFxX = 13, kFxLeft1 = 14, kFxLeft30 = 15, kFxT1 = 16, kFxT30 = 17, kFxI = 18, kFxH = 19, kFx30Stats = 20 };
+// Grr, Gss, Gtt, derivatives along r, s, t (FxScales) and sum at the Gauss
+// points, whether the element is left to FP64 (BP1.0, BP3.0), the largest value
+// after the projection along t (BP1.0, BP3.0) and after the interpolation along
+// s, the largest scale of a transposed line (as 63 - its scale-up) and of the
+// direction of one that is not zero (N = 1), the directions' scales (fx_below).
+enum {
+    kFxW = 8, kFxG = 9, kFxU = 12, kFxX = 15, kFxLeft1 = 16, kFxLeft30 = 17, kFxT1 = 18, kFxT30 = 19, kFxI = 20, kFxH = 21,
+    kFxE = 22, kFxB = 23, kFx30Stats = 24
+};
 
 // A line of Q values at from(l), contracted, its outputs to put(l, y).
 template <int P, int Q, int SIG, int OFF, class L, class F>
@@ -459,6 +464,7 @@ __device__ __forceinline__ void bp30_fx_block(unsigned char *smem_raw, int64_t e
     constexpr int n = C::n, m = C::m, nn = C::nn, mm = C::mm, NP = C::NP, MP = C::MP, S = C::S, K = kFx30Stats, QB = kFxBits30, qb = fx_qbits30(N);
     constexpr int oI = fold_offset(N, kFoldI), oIT = fold_offset(N, kFoldIT);
     constexpr int oDt = fold_offset(N, kFoldDt), oDtT = fold_offset(N, kFoldDtT);
+    constexpr bool EXACT = N == 1;  // FP64 may interpolate and differentiate without an error
     const int el = threadIdx.x / mm, r = threadIdx.x - el * mm;
     const bool act = el < nel;
     const int u = r % m, v = r / m;
@@ -553,47 +559,67 @@ __device__ __forceinline__ void bp30_fx_block(unsigned char *smem_raw, int64_t e
 
     // derivatives along r (A -> B), s (A -> C) and t (A -> D)
     if (act) {
-        int most = fx_derivative<B3, m, oDt, 0>(A, B, u, v);
-        most = max(most, fx_derivative<B3, m, oDt, 1>(A, Cx, u, v));
-        most = max(most, fx_derivative<B3, m, oDt, 2>(A, D, u, v));
-        fx_element_max<mm>(st + kFxU, (unsigned)most);
+        const int mr = fx_derivative<B3, m, oDt, 0>(A, B, u, v), ms = fx_derivative<B3, m, oDt, 1>(A, Cx, u, v),
+                  mt = fx_derivative<B3, m, oDt, 2>(A, D, u, v);
+        fx_element_max<mm>(st + kFxU, (unsigned)mr);
+        fx_element_max<mm>(st + kFxU + 1, (unsigned)ms);
+        fx_element_max<mm>(st + kFxU + 2, (unsigned)mt);
     }
     __syncthreads();
 
     // chain rule at the points of column (a=u, b=v)
     int basez = 0;
     if (act) {
-        int kg = (int)(max(st[kFxG], max(st[kFxG + 1], st[kFxG + 2])) >> 20) - 1022;
-        bool left = kg > 800 || kg < -800 || kq + kg > 800 || kq + kg < -800;
-        const int sh = max(0, QB - 32 - fx_top((int)st[kFxU]));
-        basez = kq - qb + t3 + c_fxd[N].tau[kFoldDt] - sh + 2 + kg + c_fxd[N].tau[kFoldDtT];
+        const FxScales<QB> Z(st + kFxG);
+        const int kg = Z.kg;
+        const bool left = Z.bad || kq + kg > 800 || kq + kg < -800;
+        basez = kq - qb + t3 + c_fxd[N].tau[kFoldDt] - Z.sh + 2 + kg + c_fxd[N].tau[kFoldDtT];
         const int eg = kg + 1022 + wuv;
         FxRange range;
-#pragma unroll 4
-        for (int c = 0; c < m; c++) {
+        auto chain = [&](int c, auto split) {
             const int s = B3::at(u, v, c);
-            fx_chain(Ge + c * mm, MP, eg + c_fxd[N].wm[c], B[s] << sh, Cx[s] << sh, D[s] << sh, B[s], Cx[s], D[s], range);
+            fx_chain<split.value>(Ge + c * mm, MP, eg + c_fxd[N].wm[c], Z, B[s], Cx[s], D[s], B[s], Cx[s], D[s], range);
+        };
+        if (!Z.split) {
+#pragma unroll 4
+            for (int c = 0; c < m; c++) chain(c, std::false_type());
+        } else {
+#pragma unroll 1
+            for (int c = 0; c < m; c++) chain(c, std::true_type());
         }
         if (left || range.left()) st[kFxLeft30] = 1;
+        if (r == 0) st[kFxB] = Z.below();
     }
     __syncthreads();
 
     // transposes, in place; ln: each line's scale
     if (act) {
-        const int hr = fx_transpose<B3, m, oDtT, QB, 0>(B, u, v), hs = fx_transpose<B3, m, oDtT, QB, 1>(Cx, u, v),
-                  ht = fx_transpose<B3, m, oDtT, QB, 2>(D, u, v);
+        const unsigned below = st[kFxB];
+        const int hr = fx_transpose<B3, m, oDtT, QB, 0, EXACT>(B, u, v) + fx_below(below, 0),
+                  hs = fx_transpose<B3, m, oDtT, QB, 1, EXACT>(Cx, u, v) + fx_below(below, 1),
+                  ht = fx_transpose<B3, m, oDtT, QB, 2, EXACT>(D, u, v) + fx_below(below, 2);
         ln[r] = hr;
         ln[mm + r] = hs;
         ln[2 * mm + r] = ht;
-        fx_element_max<mm>(st + kFxH, (unsigned)(63 - __vimin3_s32(hr, hs, ht)));
+        const int h = __vimin3_s32(hr, hs, ht);
+        if (!EXACT || h < kFxZeroLine) fx_element_max<EXACT ? 1 : mm>(st + kFxH, (unsigned)(63 - h));
+        if (EXACT) {
+            const int unit = __vimin3_s32(hr < kFxZeroLine ? fx_below(below, 0) : 63, hs < kFxZeroLine ? fx_below(below, 1) : 63,
+                                          ht < kFxZeroLine ? fx_below(below, 2) : 63);
+            atomicMax(st + kFxE, (unsigned)(63 - unit));
+        }
     }
     __syncthreads();
 
     // column: the three directions and lambda wJ q, aligned (-> D)
     int zs = 0;
     if (act) {
-        const int hm = 63 - (int)st[kFxH];  // every line is brought to the largest scale among them
+        // every line is brought to the largest scale among them (N = 1: that are not zero)
+        const int hm = (EXACT && st[kFxH] == 0) ? QB - 32 : 63 - (int)st[kFxH];
         basez -= hm;
+        // lines are known to a unit of their direction's scale: the largest
+        // must not lie far below that of the largest that is not zero
+        const bool lost = EXACT && st[kFxH] != 0 && st[kFxH] + kFxRange < st[kFxE];
         int el2 = 0;  // |lambda| < 2^el2
         if (lambda != 0.0) el2 = ((__double2hiint(lambda) >> 20) & 0x7ff) - 1022;
         const int delta = kq - qb + t3 + kw + el2 - basez;  // scale of the mass term over the other's
@@ -601,13 +627,14 @@ __device__ __forceinline__ void bp30_fx_block(unsigned char *smem_raw, int64_t e
         const int ms = min(63, max(0, -delta)), bw = kw + el2 + 1022 + wuv, ht = ln[2 * mm + r] - hm + zs;
         bool left = el2 > 200 || el2 < -200 || delta > 63 || kw > 800 || kw < -800 || kq + kw > 800 || kq + kw < -800;
         if (lambda == 0.0) left = false;
+        left = left || lost;
         FxMost most;
         int far = 0, least = 0;
 #pragma unroll 4
         for (int c = 0; c < m; c++) {
             const int s = B3::at(u, v, c);
-            long long x = (B[s] >> min(63, ln[v + m * c] - hm + zs)) +
-                          (Cx[s] >> min(63, ln[mm + u + m * c] - hm + zs)) + (D[s] >> min(63, ht));
+            long long x = fx_shr(B[s], ln[v + m * c] - hm + zs) + fx_shr(Cx[s], ln[mm + u + m * c] - hm + zs) +
+                          fx_shr(D[s], ht);
             if (lambda != 0.0) {
                 const double wj = lambda * __ldg(Ge + 6 * MP + c * mm);
                 const int e = (__double2hiint(wj) >> 20) & 0x7ff, d = bw + c_fxd[N].wm[c] - e;

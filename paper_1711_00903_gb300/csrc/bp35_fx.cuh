@@ -9,7 +9,7 @@
 //      field they are far below the bound ||D|| max|q|);
 //   3. chain rule: the factors without their quadrature weights' powers of
 //      two, scaled by the element's largest diagonal factor to 62 bits, times
-//      the derivatives;
+//      the derivatives; on flat elements a scale for each direction (FxScales);
 //   4. transposes, each line scaled up by its own largest value, the weights
 //      in the operator (fx.cuh);
 //   5. the three directions aligned to the largest scale at a node, summed,
@@ -28,7 +28,10 @@
 // a node whose result is made of values all far smaller than the element's
 // largest (in FP64 it keeps digits that the element's scale cuts off), a
 // point whose factors are far smaller than the element's largest, or an
-// off-diagonal factor above every diagonal one (G not positive definite).
+// off-diagonal factor above every diagonal one (G not positive definite).  At
+// two and three points a line, where FP64 takes the derivative of a constant
+// (at two of any line) without an error, also a node whose lines hold far less
+// than the scale of the directions that reach it.
 // The choice is made element by element, so a result does not depend on the
 // other elements of the block.  Of a smooth field that vanishes on the faces
 // of a box, the elements along the box's edges go this way (0.6 % of 32^3
@@ -45,8 +48,9 @@ namespace {
 template <int N, int EPB_>
 struct Fx35Layout : Bp35Layout<double, N, EPB_> {
     using L = Bp35Layout<double, N, EPB_>;
-    // per element: max q, max Grr, Gss, Gtt, max derivative, left out, values below a unit
-    static constexpr int kStats = 7;
+    // per element: max q; max Grr, Gss, Gtt; max derivative along r, s, t; left out; values below a unit;
+    // the directions' scales (fx_below)
+    static constexpr int kStats = 10;
     // boxes, then a word per line, then the statistics
     static constexpr int off_e = L::bytes;
     static constexpr int off_s = off_e + EPB_ * 3 * L::nn * 4;
@@ -138,6 +142,7 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
     using C = Fx35Layout<N, EPB_>;
     using B = typename C::B;
     constexpr int n = C::n, nn = C::nn, NP = C::NP, QB = fx_bits35(N), K = C::kStats;
+    constexpr bool EXACT = n <= 3;  // FP64 lines may make no error
     constexpr int UC = 4;  // nodes of a column taken at a time (whole columns spill)
     constexpr int oD = fold_offset(N, kFoldD), oDT = fold_offset(N, kFoldDT);
     const int el = threadIdx.x / nn, r = threadIdx.x - el * nn;
@@ -187,7 +192,7 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
 #pragma unroll
             for (int k = 0; k < n; k++) bad = bad || __double2loint(qv[k]) != 0;
         }
-        if (bad) st[5] = 1;
+        if (bad) st[7] = 1;
         int most = 0;  // largest shift of a value that is not zero
 #pragma unroll
         for (int k = 0; k < n; k++) {
@@ -195,21 +200,21 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
             if ((fx_abs_hi(qv[k]) | __double2loint(qv[k])) != 0) most = max(most, sq);
             box[B::at(u, v, k)] = fx_from_double<qb>(qv[k], sq);
         }
-        if (most >= qb) st[6] = 1;
+        if (most >= qb) st[8] = 1;
     }
     __syncthreads();
 
     // derivatives along r and s to boxes 1 and 2, then along t in place in
     // box 0; ln: each line's largest value
-    int m = 0;
     if (act) {
-        m = fx_derivative<B, n, oD, 0, true>(box, box + B::size, u, v, ln + r);
-        m = max(m, fx_derivative<B, n, oD, 1, true>(box, box + 2 * B::size, u, v, ln + nn + r));
+        const int mr = fx_derivative<B, n, oD, 0, true>(box, box + B::size, u, v, ln + r),
+                  ms = fx_derivative<B, n, oD, 1, true>(box, box + 2 * B::size, u, v, ln + nn + r);
+        fx_element_max<nn>(st + 4, (unsigned)mr);
+        fx_element_max<nn>(st + 5, (unsigned)ms);
     }
     __syncthreads();
     if (act) {
-        m = max(m, fx_derivative<B, n, oD, 2, true>(box, box, u, v, ln + 2 * nn + r));
-        fx_element_max<nn>(st + 4, (unsigned)m);
+        fx_element_max<nn>(st + 6, (unsigned)fx_derivative<B, n, oD, 2, true>(box, box, u, v, ln + 2 * nn + r));
         // the diagonal factors' largest exponents, without the weights
         // (prefetched into L2 when the block began)
         int gm[3] = {0, 0, 0};
@@ -228,44 +233,69 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
     // chain rule at the nodes of column (i=u, j=v)
     int base = 0;
     if (act) {
-        int kd[3];  // diagonal factors without weights < 2^kg
-#pragma unroll
-        for (int d = 0; d < 3; d++) kd[d] = (int)(st[1 + d] >> 20) - 1022;
-        const int kg = __vimax3_s32(kd[0], kd[1], kd[2]);
-        bool bad = kg > 800 || kg < -800 || kq + kg > 800 || kq + kg < -800;
-        // a node is held to the element's scale by its largest line
+        const FxScales<QB> S(st + 1);
+        const int kg = S.kg;
+        bool bad = S.bad || kq + kg > 800 || kq + kg < -800;
+        // a node is held to the element's scale by its largest line; kd: diagonal factors without weights < 2^kd
+        const int most = (int)(max(st[1], max(st[2], st[3])) >> 20);
+        auto kd = [&](int d) { return (int)(st[1 + d] >> 20) - most; };
         const int need = qb - 32 - kFxRange;  // bits of a line's high word, with its factor at the largest
         const int lt = ln[2 * nn + r];
-        if (fx_top(lt) + kd[2] - kg < need) {
+        if (fx_top(lt) + kd(2) < need) {
 #pragma unroll 1
             for (int k = 0; k < n; k++)
-                if (fx_top(ln[v + n * k]) + kd[0] - kg < need && fx_top(ln[nn + u + n * k]) + kd[1] - kg < need)
-                    bad = bad || !fx35_held(ln, G + (e0 + el) * 7 * NP, n, u, v, k, c_fxd[N].wn, kg, need, st[6] != 0);
+                if (fx_top(ln[v + n * k]) + kd(0) < need && fx_top(ln[nn + u + n * k]) + kd(1) < need)
+                    bad = bad || !fx35_held(ln, G + (e0 + el) * 7 * NP, n, u, v, k, c_fxd[N].wn, most - 1022, need,
+                                            st[8] != 0);
         }
-        const int sh = QB - 32 - fx_top((int)st[4]);
-        base = kq - qb + c_fxd[N].tau[kFoldD] - sh + 2 + kg + c_fxd[N].tau[kFoldDT];
+        base = kq - qb + c_fxd[N].tau[kFoldD] - S.sh + 2 + kg + c_fxd[N].tau[kFoldDT];
         const int eg = kg + 1022 + wuv;
         FxRange range;
-#pragma unroll(UC)
-        for (int k = 0; k < n; k++) {
+        auto chain = [&](int k, auto split) {
             const int s = B::at(u, v, k);
             long long *rr = box + B::size + s, *ss = rr + B::size, *tt = box + s;
-            fx_chain(Ge + k * nn, NP, eg + c_fxd[N].wn[k], *rr << sh, *ss << sh, *tt << sh, *rr, *ss, *tt, range);
+            fx_chain<split.value>(Ge + k * nn, NP, eg + c_fxd[N].wn[k], S, *rr, *ss, *tt, *rr, *ss, *tt, range);
+        };
+        if (!S.split) {
+#pragma unroll(UC)
+            for (int k = 0; k < n; k++) chain(k, std::false_type());
+        } else {
+#pragma unroll 1
+            for (int k = 0; k < n; k++) chain(k, std::true_type());
         }
-        if (bad || range.left()) st[5] = 1;
+        if (bad || range.left()) st[7] = 1;
+        if (r == 0) st[9] = S.below();
     }
     __syncthreads();
 
     // transposes, in place; ln: each line's exponent
     if (act) {
-        ln[r] = -fx_transpose<B, n, oDT, QB, 0>(box + B::size, u, v);
-        ln[nn + r] = -fx_transpose<B, n, oDT, QB, 1>(box + 2 * B::size, u, v);
-        ln[2 * nn + r] = -fx_transpose<B, n, oDT, QB, 2>(box, u, v);
+        ln[r] = -fx_transpose<B, n, oDT, QB, 0, EXACT>(box + B::size, u, v) - fx_below(st[9], 0);
+        ln[nn + r] = -fx_transpose<B, n, oDT, QB, 1, EXACT>(box + 2 * B::size, u, v) - fx_below(st[9], 1);
+        ln[2 * nn + r] = -fx_transpose<B, n, oDT, QB, 2, EXACT>(box, u, v) - fx_below(st[9], 2);
     }
     __syncthreads();
 
+    // a node's lines are known to a unit of their directions' scale: its
+    // largest must not lie far below that of the largest that is not zero
+    if constexpr (EXACT) {
+        if (act) {
+            const unsigned below = st[9];
+            const int et = ln[2 * nn + r];
+#pragma unroll
+            for (int k = 0; k < n; k++) {
+                const int a = ln[v + n * k], b = ln[nn + u + n * k];
+                const int unit = __vimax3_s32(a > -kFxZeroLine ? -fx_below(below, 0) : -kFxZeroLine,
+                                              b > -kFxZeroLine ? -fx_below(below, 1) : -kFxZeroLine,
+                                              et > -kFxZeroLine ? -fx_below(below, 2) : -kFxZeroLine);
+                if (unit > -kFxZeroLine && __vimax3_s32(et, a, b) < unit - kFxRange) st[7] = 1;
+            }
+        }
+        __syncthreads();
+    }
+
     double dot = 0.0;  // p . Ap of the thread's column
-    if (act && st[5] == 0) {
+    if (act && st[7] == 0) {
         const int64_t g0 = (e0 + el) * NP + r;
         const double *qe = PCG ? p : q;
         const int et = ln[2 * nn + r];
@@ -274,7 +304,7 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
             const int s = B::at(u, v, k);
             const int a = ln[v + n * k], b = ln[nn + u + n * k], d = __vimax3_s32(et, a, b);
             const long long sum =
-                (box[s] >> (d - et)) + (box[B::size + s] >> (d - a)) + (box[2 * B::size + s] >> (d - b));
+                fx_shr(box[s], d - et) + fx_shr(box[B::size + s], d - a) + fx_shr(box[2 * B::size + s], d - b);
             double w = fx_to_double(sum, base + d + wuv + c_fxd[N].wn[k]);
             const double qk = qe[g0 + k * nn];
             if (lambda != 0.0) w = fma(lambda, __ldg(Ge + 6 * NP + k * nn) * qk, w);
@@ -283,7 +313,7 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
         }
     }
     for (int e = 0; e < nel; e++)
-        if (stats[e * K + 5] != 0) {  // the same for every thread
+        if (stats[e * K + 7] != 0) {  // the same for every thread
             const double d = bp35_element64(reinterpret_cast<double *>(smem_raw), n, oD, oDT, G + (e0 + e) * 7 * NP,
                                             lambda, (PCG ? p : q) + (e0 + e) * NP, Aq + (e0 + e) * NP);
             if (PCG) dot += d;

@@ -71,49 +71,134 @@ __device__ __forceinline__ int fx_derivative(const long long *from, long long *t
     return max(hi, ~lo);
 }
 
+// What fx_transpose<.., ZERO> returns for a line of zeros: more than any shift.
+constexpr int kFxZeroLine = 1000;
+
 // The transpose along a line of direction D, in place, the line first scaled
 // up to QB bits; returns the shift.
-template <class B, int n, int OFF, int QB, int D>
+template <class B, int n, int OFF, int QB, int D, bool ZERO = false>
 __device__ __forceinline__ int fx_transpose(long long *box, int u, int v) {
     long long x[n];
 #pragma unroll
     for (int l = 0; l < n; l++) x[l] = box[fx_at<B, D>(l, u, v)];
     const int h = max(0, QB - 32 - fx_top(fx_line_max(x)));
+    if (ZERO) {
+        long long any = 0;
+#pragma unroll
+        for (int l = 0; l < n; l++) any |= x[l];
+        if (any == 0) return kFxZeroLine;
+    }
 #pragma unroll
     for (int l = 0; l < n; l++) x[l] <<= h;
     fx_apply<n, n, -1, OFF>(x, [&](int l, long long y) { box[fx_at<B, D>(l, u, v)] = y; });
     return h;
 }
 
-// What the factors of a thread's points showed: a factor above the element's
-// largest diagonal one (or not finite), a point whose diagonal factors are
-// all far below it, a negative diagonal factor.
+// x >> s for any s >= 0 (above 63: the sign).
+__device__ __forceinline__ long long fx_shr(long long x, int s) {
+    asm("shr.s64 %0, %0, %1;" : "+l"(x) : "r"(s));
+    return x;
+}
+
+// Scales of an element's three directions.  With one scale for all factors, a
+// flat element's small ones would keep few bits (aspect 1000: 42 of 62), and
+// the result none where the derivative across the thin direction is zero.
+// So where the directions' e_d, half the exponents of their largest diagonal
+// factors, differ by more than kFxAlike, each direction has its own scale 2^e_d: the factors are held as G_ab / 2^(e_a + e_b),
+// below 1 for a positive definite G, and the derivatives as d_b 2^(e_b).
+// Elsewhere one scale serves.  (The kernels have a loop for each: in one, the
+// directions' shifts spilled at N = 7.)
+constexpr int kFxAlike = 2;
+// Directions further apart than this leave the element to FP64: up to here
+// shifting a value to another direction's scale drops no bit that it holds.
+constexpr int kFxApart = 28;
+
+// slot: the element's largest diagonal factors without weights (high words),
+// then the largest derivatives (high words), along r, s, t.
+template <int QB>
+struct FxScales {
+    const unsigned *slot;
+    int kg;      // factors < 2^kg; split: 2 e of the direction with the largest
+    int sh;      // the derivatives' common shift up
+    bool split;  // a scale for each direction
+    bool bad;    // out of range
+
+    __device__ __forceinline__ int half(int d) const { return ((int)(slot[d] >> 20) - 1021) >> 1; }
+    // Shift of direction d's line scales, and of its factors, below the largest's.
+    __device__ __forceinline__ int below(int d) const { return split ? (kg >> 1) - half(d) : 0; }
+    // All three in one word, for a later phase (fx_below).
+    __device__ __forceinline__ unsigned below() const {
+        return split ? (unsigned)(below(0) & 255) | (unsigned)(below(1) & 255) << 8 | (unsigned)(below(2) & 255) << 16 : 0u;
+    }
+    __device__ __forceinline__ int up(int d) const { return max(0, QB - 32 - fx_top((int)slot[3 + d])); }
+
+    __device__ __forceinline__ explicit FxScales(const unsigned *slot_) : slot(slot_) {
+        const int e0 = half(0), e1 = half(1), e2 = half(2), most = __vimax3_s32(e0, e1, e2),
+                  apart = most - __vimin3_s32(e0, e1, e2);
+        split = apart > kFxAlike;
+        kg = split ? 2 * most : (int)(max(slot[0], max(slot[1], slot[2])) >> 20) - 1022;
+        sh = __vimin3_s32(up(0) + below(0), up(1) + below(1), up(2) + below(2));
+        bad = apart > kFxApart || kg > 800 || kg < -800;
+    }
+    // The derivatives on one scale with their directions' 2^e, and the factors' shifts.
+    __device__ __forceinline__ void scale(long long &dr, long long &ds, long long &dt, int (&s)[6]) const {
+        const int a = below(0), b = below(1), c = below(2), ur = up(0), us = up(1), ut = up(2);
+        dr = fx_shr(dr << ur, ur + a - sh);
+        ds = fx_shr(ds << us, us + b - sh);
+        dt = fx_shr(dt << ut, ut + c - sh);
+        s[0] -= 2 * a;
+        s[1] -= a + b;
+        s[2] -= a + c;
+        s[3] -= 2 * b;
+        s[4] -= b + c;
+        s[5] -= 2 * c;
+    }
+};
+
+__device__ __forceinline__ int fx_below(unsigned word, int d) { return (int)(word >> (8 * d)) & 255; }
+
+// What the factors of a thread's points showed: a factor above the scale
+// (or not finite), a point whose diagonal factors are all far below it, a
+// negative diagonal factor, and (split) the diagonal factor furthest below.
+// 62 bits hold one exactly down to kFxExact bits below its scale.
+constexpr int kFxExact = 9;
 struct FxRange {
-    int least = 0, far = 0, sign = 0;
-    __device__ __forceinline__ bool left() const { return least < 0 || far > kFxRange || sign < 0; }
+    int least = 0, far = 0, sign = 0, deep = 0;
+    __device__ __forceinline__ bool left() const { return least < 0 || far > kFxRange || sign < 0 || deep > kFxExact; }
 };
 
 // Chain rule at a point: (wr, ws, wt) = G (dr, ds, dt) / 2^64, the factors at
-// g[h plane], h = 0..5, scaled to 62 bits by eg: the largest diagonal factor's
-// biased exponent with the point's weights.
-__device__ __forceinline__ void fx_chain(const double *g, int plane, int eg, long long dr, long long ds, long long dt,
-                                         long long &wr, long long &ws, long long &wt, FxRange &range) {
+// g[h plane], h = 0..5, scaled to 62 bits by eg: the scale's biased exponent
+// (S.kg) with the point's weights; the derivatives as the lines left them.
+template <bool SPLIT, int QB>
+__device__ __forceinline__ void fx_chain(const double *g, int plane, int eg, const FxScales<QB> &S, long long dr,
+                                         long long ds, long long dt, long long &wr, long long &ws, long long &wt,
+                                         FxRange &range) {
     double f[6];
 #pragma unroll
     for (int h = 0; h < 6; h++) f[h] = __ldg(g + h * plane);
     range.sign |= __double2hiint(f[0]) | __double2hiint(f[3]) | __double2hiint(f[5]);
-    const int s0 = eg - (__double2hiint(f[0]) >> 20), s3 = eg - (__double2hiint(f[3]) >> 20),
-              s5 = eg - (__double2hiint(f[5]) >> 20), s1 = eg - ((__double2hiint(f[1]) >> 20) & 0x7ff),
-              s2 = eg - ((__double2hiint(f[2]) >> 20) & 0x7ff), s4 = eg - ((__double2hiint(f[4]) >> 20) & 0x7ff);
-    range.least = __vimin3_s32(range.least, __vimin3_s32(s0, s1, s2), __vimin3_s32(s3, s4, s5));
-    range.far = max(range.far, __vimin3_s32(s0, s3, s5));
+    int s[6];  // (a negative diagonal factor leaves the element to FP64 whatever its s)
+#pragma unroll
+    for (int h = 0; h < 6; h++)
+        s[h] = eg - ((h == 0 || h == 3 || h == 5) ? __double2hiint(f[h]) >> 20 : (__double2hiint(f[h]) >> 20) & 0x7ff);
+    if (SPLIT) {
+        S.scale(dr, ds, dt, s);
+        range.deep = max(range.deep, __vimax3_s32(s[0], s[3], s[5]));
+    } else {
+        dr <<= S.sh;
+        ds <<= S.sh;
+        dt <<= S.sh;
+    }
+    range.least = __vimin3_s32(range.least, __vimin3_s32(s[0], s[1], s[2]), __vimin3_s32(s[3], s[4], s[5]));
+    range.far = max(range.far, __vimin3_s32(s[0], s[3], s[5]));
     int h[6], l[6];
-    fx_diagonal(f[0], s0, h[0], l[0]);
-    fx_off_diagonal(f[1], s1, h[1], l[1]);
-    fx_off_diagonal(f[2], s2, h[2], l[2]);
-    fx_diagonal(f[3], s3, h[3], l[3]);
-    fx_off_diagonal(f[4], s4, h[4], l[4]);
-    fx_diagonal(f[5], s5, h[5], l[5]);
+    fx_diagonal(f[0], s[0], h[0], l[0]);
+    fx_off_diagonal(f[1], s[1], h[1], l[1]);
+    fx_off_diagonal(f[2], s[2], h[2], l[2]);
+    fx_diagonal(f[3], s[3], h[3], l[3]);
+    fx_off_diagonal(f[4], s[4], h[4], l[4]);
+    fx_diagonal(f[5], s[5], h[5], l[5]);
     wr = fx_dot3(h[0], l[0], dr, h[1], l[1], ds, h[2], l[2], dt);
     ws = fx_dot3(h[1], l[1], dr, h[3], l[3], ds, h[4], l[4], dt);
     wt = fx_dot3(h[2], l[2], dr, h[4], l[4], ds, h[5], l[5], dt);

@@ -102,3 +102,96 @@ def test_factors_of_nearly_parallel_edges(N):
         assert np.all(abs(got - ref) <= bar)
     wj = fem.fem_mesh_geofacs(b, fem.FEM_GEO_BP1, _dev(verts)).cpu().numpy()
     np.testing.assert_array_equal(wj, got[:, 6])
+
+
+# ------------------------------------------------------------ flat elements
+
+def _along(A, u, axis):
+    return np.moveaxis(np.tensordot(A, u, axes=(1, axis)), 0, axis)
+
+
+def _all3(A, u):
+    return _along(A, _along(A, _along(A, u, 3), 2), 1)
+
+
+def _symmetric(A, s):
+    A = A.astype(LD)
+    return (A + s * A[::-1, ::-1]) / 2
+
+
+def _stiff(T, G, u, d):
+    """T G d + 0.37 wJ u of the derivatives d (along r, s, t)."""
+    g = G.reshape(-1, 7, *u.shape[1:])
+    w = [sum(g[:, k] * x for k, x in zip(row, d)) for row in ((0, 1, 2), (1, 3, 4), (2, 4, 5))]
+    return _along(T, w[0], 3) + _along(T, w[1], 2) + _along(T, w[2], 1) + LD(0.37) * g[:, 6] * u
+
+
+def _folded(A):
+    """Absolute values of an operator as even-odd folded lines add them up."""
+    return abs(A) + abs(A[:, ::-1])
+
+
+def _flat_reference(op, t, G, q, exact):
+    """The operator and the bound 2 (1.5 n + 17) 2^-53 |D^T| |G| |d| of FP64
+    lines folded even-odd (n / 2 + 3 roundings a contraction, 8 in the chain
+    rule and the sums), with |d| the derivatives themselves along the directions
+    in `exact` (FP64 takes them without an error of the field's size) and |D|
+    |q| along the others."""
+    n = t["D"].shape[0]
+    I, D = _symmetric(t["I"], 1), _symmetric(t["D" if op == "bp35" else "Dt"], -1)
+    u, G = q.astype(LD).reshape(-1, n, n, n), G.astype(LD)
+    if op == "bp30":
+        u = _all3(I, u)
+    d = [_along(D, u, a) for a in (3, 2, 1)]
+    m = [abs(x) if a in exact else _along(_folded(D), abs(u), 3 - a) for a, x in enumerate(d)]
+    ref, bar = _stiff(D.T, G, u, d), _stiff(_folded(D.T), abs(G), abs(u), m)
+    if op == "bp30":
+        ref, bar = _all3(I.T.copy(), ref), _all3(_folded(I.T), bar)
+    chain = 1.5 if op == "bp35" else 4.5
+    return ref.reshape(q.shape), (2 * (chain * n + 17) * U * bar).reshape(q.shape)
+
+
+def _flat_fields(rng, n, thin):
+    """Constant across the thin direction; constant; with a slope of 1 to 1e-9
+    across the thin direction; random; zero but for a face."""
+    axis = 3 - thin
+    shape = [8, n, n, n]
+    shape[axis] = 1
+    flat = np.broadcast_to(rng.uniform(-1, 1, shape), (8, n, n, n))
+    x = np.linspace(0, 1, n).reshape([-1 if a == axis else 1 for a in range(4)])
+    q = flat + np.array([0, 0, 1, 1e-3, 1e-6, 1e-9, 0, 0]).reshape(8, 1, 1, 1) * x
+    q[1] = 0.7
+    q[6] = rng.uniform(-1, 1, (n, n, n))
+    q[7] = 0.0
+    q[7, 0] = rng.uniform(-1, 1, (n, n))
+    return np.ascontiguousarray(q.reshape(8, -1))
+
+
+@pytest.mark.parametrize("op,N", [("bp35", 1), ("bp35", 2), ("bp35", 3), ("bp35", 7), ("bp30", 1), ("bp30", 2),
+                                  ("bp30", 7)])
+@pytest.mark.parametrize("thin", [0, 1, 2])
+def test_flat_elements_keep_the_small_factors(op, N, thin):
+    """Each node within the error that an evaluation in FP64 may have, on
+    axis-aligned and slightly skewed elements of aspect 1 to 1e6 (and a long
+    one), where the smallest factors are aspect^-2 of the largest.  FP64 takes
+    the derivative of a constant line without an error at two and three points
+    (of any line at two)."""
+    fem, rng = _fem(), np.random.default_rng(100 * N + thin)
+    b = fem.fem_basis_setup(N)
+    t = fem.fem_basis_host_tables(N)
+    kind, apply = (fem.FEM_GEO_BP35, fem.fem_bp35_apply) if op == "bp35" else (fem.FEM_GEO_BP30, fem.fem_bp30_apply)
+    for aspect in (1, 10, 100, 1e3, 1e4, 1e6, 1e9, 1e-3):
+        scale = np.ones(3)
+        scale[thin] = 1 / aspect
+        for skew in (0, 0.05):
+            verts = np.ascontiguousarray((BOX + skew * rng.uniform(-1, 1, (8, 8, 3))) * scale)
+            q = _flat_fields(rng, N + 1, thin)
+            G = fem.fem_mesh_geofacs(b, kind, _dev(verts))
+            got = apply(b, G, 0.37, _dev(q)).cpu().numpy()
+            for rows, exact in ((slice(0, 2), (thin,)), (slice(2, 8), ())):
+                if op == "bp35" and N == 1:
+                    exact = (0, 1, 2)
+                elif N > (2 if op == "bp35" else 1):
+                    exact = ()
+                ref, bar = _flat_reference(op, t, G.cpu().numpy()[rows], q[rows], exact)
+                assert np.all(abs(got[rows] - ref) <= bar)
