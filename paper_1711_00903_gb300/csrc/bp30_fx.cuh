@@ -19,7 +19,7 @@
 // BP1.0 computed beside BP3.0 takes the same steps on the same numbers as
 // alone, and BP3.0 the same with and without it: equal bits.
 //
-// An element goes through FP64 instead (bp1_element64, bp30_element64) when
+// An element goes through FP64 instead (bp1_left64, bp30_left64) when
 // its values are not finite or extreme, when one of its eight octants holds
 // no value near its largest (the FP64 result there would keep digits that
 // the element's scale cuts off), when a point's factors are far below the
@@ -160,6 +160,11 @@ __device__ __forceinline__ void fx30_load(double (&qv)[N + 1], int64_t g0, int r
     }
 }
 
+// High word (so: sign) of a factor that has to be positive, read ahead with the
+// field: an element of a left-handed mesh has them all negative, and is left
+// to FP64 before its contractions.
+__device__ __forceinline__ int fx30_sign(const double *g) { return __ldg(reinterpret_cast<const int *>(g) + 1); }
+
 // The element's scale from its octants: |q| < 2^kq; left: the element is not
 // held to one scale.
 template <int N>
@@ -216,108 +221,64 @@ __device__ __forceinline__ int fx1_exponent(const unsigned *st) {
            (int)(st[kFxW] >> 20) - 1022;
 }
 
-// Algorithm 3 in FP64 on one element by the whole block, sizes at run time
-// (fx_line64); smem: at least 2 m^3 doubles (rows of m, or m + 1 for even m).
-__device__ __noinline__ void bp1_element64(double *smem, int n, int oI, int oIT, const double *wJ, const double *q,
-                                           double *Mq) {
-    const int m = n + 1, mm = m * m, nn = n * n, NP = nn * n, sj = m | 1, sk = sj * m;
-    double *X = smem, *Y = smem + sk * m;
-    __syncthreads();  // the shared memory is free
-    for (int t = threadIdx.x; t < NP; t += blockDim.x) X[t % n + sj * ((t / n) % n) + sk * (t / nn)] = q[t];
-    __syncthreads();
-    for (int t = threadIdx.x; t < nn; t += blockDim.x) {
-        const int o = sj * (t % n) + sk * (t / n);
-        fx_line64(X + o, 1, Y + o, 1, m, n, 1, oI);
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < m * n; t += blockDim.x) {
-        const int o = t % m + sk * (t / m);
-        fx_line64(Y + o, sj, X + o, sj, m, n, 1, oI);
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < mm; t += blockDim.x) {
-        const int o = t % m + sj * (t / m);
-        double g[kMaxQ];
-        fx_line64(X + o, sk, g, 1, m, n, 1, oI);
-        for (int c = 0; c < m; c++) g[c] *= wJ[t + c * mm];
-        fx_line64(g, 1, X + o, sk, n, m, 1, oIT);
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < m * n; t += blockDim.x) {
-        const int o = t % m + sk * (t / m);
-        fx_line64(X + o, sj, Y + o, sj, n, m, 1, oIT);
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nn; t += blockDim.x)
-        fx_line64(Y + sj * (t % n) + sk * (t / n), 1, Mq + t * n, 1, n, m, 1, oIT);
+// A line of doubles at from(l), contracted in FP64, its outputs to put(l, y).
+template <int P, int Q, int SIG, int OFF, class L, class F>
+__device__ __forceinline__ void fx_from64(L &&from, F &&put) {
+    double x[Q];
+#pragma unroll
+    for (int l = 0; l < Q; l++) x[l] = from(l);
+    fx_line64<P, Q, SIG, OFF>(x, put);
 }
 
-// Algorithm 5 in FP64 on one element by the whole block (at least m^2
-// threads); smem: at least 3 m^3 doubles as above.
-__device__ __noinline__ void bp30_element64(double *smem, int n, int oI, int oIT, int oDt, int oDtT, const double *G,
-                                            double lambda, const double *q, double *Aq) {
-    const int m = n + 1, mm = m * m, MP = mm * m, nn = n * n, NP = nn * n, sj = m | 1, sk = sj * m, size = sk * m;
-    double *A = smem, *B = A + size, *C = B + size;
-    __syncthreads();  // the shared memory is free
-    for (int t = threadIdx.x; t < NP; t += blockDim.x) B[t % n + sj * ((t / n) % n) + sk * (t / nn)] = q[t];
+// In FP64, of the block's elements for which on(e) holds: the interpolation
+// along r (box X to Y) and s (Y to X), between barriers.
+template <int N, int EPB_, class B0, class B1, class B2, class F>
+__device__ __forceinline__ void fx30_interpolate64(int nel, double *X, double *Y, int per, F &&on) {
+    constexpr int n = N + 1, m = N + 2, oI = fold_offset(N, kFoldI);
+    for_tasks<n * n, EPB_>(nel, [&](int e, int t) {
+        if (!on(e)) return;
+        const double *x = X + e * per;
+        double *y = Y + e * per;
+        const int j = t % n, k = t / n;
+        fx_from64<m, n, 1, oI>([&](int l) { return x[B0::at(l, j, k)]; }, [&](int l, double w) { y[B1::at(l, j, k)] = w; });
+    });
     __syncthreads();
-    for (int t = threadIdx.x; t < nn; t += blockDim.x) {
-        const int o = sj * (t % n) + sk * (t / n);
-        fx_line64(B + o, 1, C + o, 1, m, n, 1, oI);
-    }
+    for_tasks<m * n, EPB_>(nel, [&](int e, int t) {
+        if (!on(e)) return;
+        const double *y = Y + e * per;
+        double *x = X + e * per;
+        const int i = t % m, k = t / m;
+        fx_from64<m, n, 1, oI>([&](int l) { return y[B1::at(i, l, k)]; }, [&](int l, double w) { x[B2::at(i, l, k)] = w; });
+    });
     __syncthreads();
-    for (int t = threadIdx.x; t < m * n; t += blockDim.x) {
-        const int o = t % m + sk * (t / m);
-        fx_line64(C + o, sj, B + o, sj, m, n, 1, oI);
-    }
+}
+
+// The projection along s (box X to Y) and r (Y to out(e, t, l, value)).
+template <int N, int EPB_, class B1, class B2, class F, class O>
+__device__ __forceinline__ void fx30_project64(int nel, const double *X, double *Y, int per, F &&on, O &&out) {
+    constexpr int n = N + 1, m = N + 2, oIT = fold_offset(N, kFoldIT);
+    for_tasks<m * n, EPB_>(nel, [&](int e, int t) {
+        if (!on(e)) return;
+        const double *x = X + e * per;
+        double *y = Y + e * per;
+        const int i = t % m, k = t / m;
+        fx_from64<n, m, 1, oIT>([&](int l) { return x[B2::at(i, l, k)]; }, [&](int l, double w) { y[B1::at(i, l, k)] = w; });
+    });
     __syncthreads();
-    const int r = threadIdx.x, u = r % m, v = r / m, oc = u + sj * v, orr = sj * u + sk * v, os = u + sk * v;
-    if (r < mm) fx_line64(B + oc, sk, A + oc, sk, m, n, 1, oI);
-    __syncthreads();
-    double ut[kMaxQ], acc[kMaxQ];
-    if (r < mm) {
-        fx_line64(A + orr, 1, B + orr, 1, m, m, -1, oDt);
-        fx_line64(A + os, sj, C + os, sj, m, m, -1, oDt);
-        fx_line64(A + oc, sk, ut, 1, m, m, -1, oDt);
-    }
-    __syncthreads();
-    if (r < mm) {
-        for (int c = 0; c < m; c++) {
-            const int s = oc + sk * c;
-            const double *g = G + r + c * mm, qr = B[s], qs = C[s], qt = ut[c];
-            B[s] = g[0] * qr + g[MP] * qs + g[2 * MP] * qt;
-            C[s] = g[MP] * qr + g[3 * MP] * qs + g[4 * MP] * qt;
-            ut[c] = g[2 * MP] * qr + g[4 * MP] * qs + g[5 * MP] * qt;
-        }
-        fx_line64(ut, 1, acc, 1, m, m, -1, oDtT);
-        if (lambda != 0.0)
-            for (int c = 0; c < m; c++) acc[c] = fma(lambda * G[6 * MP + r + c * mm], A[oc + sk * c], acc[c]);
-    }
-    __syncthreads();
-    if (r < mm) {
-        fx_line64(B + orr, 1, B + orr, 1, m, m, -1, oDtT);
-        fx_line64(C + os, sj, C + os, sj, m, m, -1, oDtT);
-    }
-    __syncthreads();
-    if (r < mm) {
-        for (int c = 0; c < m; c++) acc[c] += B[oc + sk * c] + C[oc + sk * c];
-        fx_line64(acc, 1, A + oc, sk, n, m, 1, oIT);
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < m * n; t += blockDim.x) {
-        const int o = t % m + sk * (t / m);
-        fx_line64(A + o, sj, B + o, sj, n, m, 1, oIT);
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nn; t += blockDim.x)
-        fx_line64(B + sj * (t % n) + sk * (t / n), 1, Aq + t * n, 1, n, m, 1, oIT);
+    for_tasks<n * n, EPB_>(nel, [&](int e, int t) {
+        if (!on(e)) return;
+        const double *y = Y + e * per;
+        const int j = t % n, k = t / n;
+        fx_from64<n, m, 1, oIT>([&](int l) { return y[B1::at(l, j, k)]; }, [&](int l, double w) { out(e, t, l, w); });
+    });
 }
 
 // ---------------------------------------------------------------- BP1.0
 
 // Shared memory of EPB elements: a box for q, the twice interpolated and the
 // once projected field, one for the once interpolated and the twice
-// projected, and the statistics.  (bp1_element64 needs two m^3 boxes.)
+// projected, the statistics and two flags of the block: an element is on the
+// fixed-point path; one is left to FP64.
 template <int N, int EPB_>
 struct Fx1Layout {
     static constexpr int n = N + 1, m = N + 2, nn = n * n, mm = m * m, NP = nn * n, MP = mm * m, EPB = EPB_;
@@ -326,11 +287,45 @@ struct Fx1Layout {
     using B2 = Box<m, m, n>;
     static constexpr int SA = B0::size > B2::size ? B0::size : B2::size, per = SA + B1::size;
     static constexpr int threads = ((mm * EPB + 31) / 32) * 32;
-    // the statistics lie past the boxes of either path
-    static constexpr int boxes = EPB * per * 8, boxes64 = 2 * Box<m, m, m>::size * 8;
-    static constexpr int off_stats = boxes > boxes64 ? boxes : boxes64;
-    static constexpr int smem = off_stats + EPB * kFx30Stats * 4;
+    static constexpr int off_stats = EPB * per * 8;
+    static constexpr int off_b = off_stats + EPB * kFx30Stats * 4;  // the block's flags
+    static constexpr int smem = off_b + 8;
 };
+
+// Algorithm 3 in FP64 on the elements left to it, all at once, in the boxes of
+// the fixed-point path.  A function of its own: its registers are not that path's.
+template <int N, int EPB_>
+__device__ __noinline__ void bp1_left64(unsigned char *smem_raw, int64_t e0, int nel, const double *wJ, const double *q,
+                                        double *Mq) {
+    using C = Fx1Layout<N, EPB_>;
+    using B0 = typename C::B0;
+    using B2 = typename C::B2;
+    constexpr int n = C::n, m = C::m, nn = C::nn, mm = C::mm, NP = C::NP, MP = C::MP;
+    const unsigned *stats = reinterpret_cast<const unsigned *>(smem_raw + C::off_stats);
+    double *X = reinterpret_cast<double *>(smem_raw), *Y = X + C::SA;
+    auto on = [&](int e) { return stats[e * kFx30Stats + kFxLeft1] != 0; };
+    const int el = threadIdx.x / mm, r = threadIdx.x - el * mm;
+    const bool act = el < nel && on(el);
+    __syncthreads();  // the shared memory is free
+    if (act && r < nn) {
+#pragma unroll
+        for (int k = 0; k < n; k++) X[el * C::per + B0::at(r % n, r / n, k)] = __ldg(q + (e0 + el) * NP + r + k * nn);
+    }
+    __syncthreads();
+    fx30_interpolate64<N, EPB_, B0, typename C::B1, B2>(nel, X, Y, C::per, on);
+    if (act) {
+        double *x = X + el * C::per, w[m];
+        const double *we = wJ + (e0 + el) * MP + r;
+        const int a = r % m, b = r / m;
+        fx_from64<m, n, 1, fold_offset(N, kFoldI)>([&](int l) { return x[B2::at(a, b, l)]; },
+                                                   [&](int c, double g) { w[c] = __dmul_rn(g, __ldg(we + c * mm)); });
+        fx_line64<n, m, 1, fold_offset(N, kFoldIT)>(w, [&](int l, double y) { x[B2::at(a, b, l)] = y; });
+    }
+    __syncthreads();
+    fx30_project64<N, EPB_, typename C::B1, B2>(nel, X, Y, C::per, on, [&](int e, int t, int l, double w) {
+        Mq[(e0 + e) * NP + t * n + l] = w;
+    });
+}
 
 // BP1.0 of elements [e0, e0 + nel) by the whole block (blockDim.x >=
 // Layout::threads); wJ: m^3 values per element.
@@ -349,17 +344,20 @@ __device__ __forceinline__ void bp1_fx_block(unsigned char *smem_raw, int64_t e0
     long long *boxes = reinterpret_cast<long long *>(smem_raw);
     unsigned *stats = reinterpret_cast<unsigned *>(smem_raw + C::off_stats), *st = stats + el * K;
     if (threadIdx.x == 0) prefetch_l2(wJ + e0 * MP, (long long)nel * MP * 8);
-    for (int t = threadIdx.x; t < EPB_ * K; t += blockDim.x) stats[t] = 0;
+    volatile unsigned *flag = reinterpret_cast<volatile unsigned *>(smem_raw + C::off_b);
+    for (int t = threadIdx.x; t < EPB_ * K + 2; t += blockDim.x) stats[t] = 0;  // (the flags lie behind them)
     __syncthreads();
 
     double qv[n];
     const bool col = act && r < nn;
+    const int sign = act ? fx30_sign(wJ + (e0 + el) * MP + r) : 0;
     if (col) fx30_load<N, false>(qv, (e0 + el) * NP + r, r, q, nullptr, nullptr, nullptr, st);
     __syncthreads();
     int kq = 0;
     if (act) {
         bool left;
         kq = fx30_scale<N>(st, &left);
+        left = left || sign < 0;
         if (col) {
 #pragma unroll
             for (int k = 0; k < n; k++) {
@@ -369,70 +367,70 @@ __device__ __forceinline__ void bp1_fx_block(unsigned char *smem_raw, int64_t e0
             }
         }
         if (left) st[kFxLeft1] = 1;
+        flag[left] = 1;
     }
     __syncthreads();
-
-    // interpolation along r and s
-    for_tasks<nn, EPB_>(nel, [&](int e, int t) {
-        const long long *X = boxes + e * C::per;
-        long long *Y = boxes + e * C::per + C::SA;
-        const int j = t % n, k = t / n;
-        fx_line<m, n, 1, oI>([&](int l) { return X[B0::at(l, j, k)]; }, [&](int l, long long y) { Y[B1::at(l, j, k)] = y; });
-    });
-    const int wab = act ? c_fxd[N].wm[a] + c_fxd[N].wm[b] : 0;
-    if (act) fx30_scan<N, 1>(wJ + (e0 + el) * MP + r, {0}, wab, st + kFxW);
-    __syncthreads();
-    for_tasks<m * n, EPB_>(nel, [&](int e, int t) {
-        const long long *Y = boxes + e * C::per + C::SA;
-        long long *X = boxes + e * C::per;
-        const int i = t % m, k = t / m;
-        FxMost most;
-        fx_line<m, n, 1, oI>([&](int l) { return Y[B1::at(i, l, k)]; },
-                             [&](int l, long long y) {
-                                 X[B2::at(i, l, k)] = y;
-                                 most.see(y);
-                             });
-        atomicMax(stats + e * K + kFxI, (unsigned)most.value());
-    });
-    __syncthreads();
-
-    // column (a, b): interpolation, wJ and projection along t
-    if (act) {
-        long long *X = boxes + el * C::per, w[m];
-        const int kw = (int)(st[kFxW] >> 20) - 1022, bw = kw + 1022 + wab;
-        int far = 0, least = 0;
-        const double *we = wJ + (e0 + el) * MP + r;
-        const int up = fx30_up<N>(st);
-        fx_line<m, n, 1, oI>([&](int l) { return X[B2::at(a, b, l)] << up; },
-                             [&](int c, long long g) {
-                                 w[c] = fx30_mass(__ldg(we + c * mm), bw + c_fxd[N].wm[c], g, far, least);
-                             });
-        FxMost most;
-        fx_apply<n, m, 1, oIT>(w, [&](int l, long long y) {
-            X[B2::at(a, b, l)] = y;
-            most.see(y);
+    if (flag[0] != 0) {
+        // interpolation along r and s
+        for_tasks<nn, EPB_>(nel, [&](int e, int t) {
+            const long long *X = boxes + e * C::per;
+            long long *Y = boxes + e * C::per + C::SA;
+            const int j = t % n, k = t / n;
+            fx_line<m, n, 1, oI>([&](int l) { return X[B0::at(l, j, k)]; }, [&](int l, long long y) { Y[B1::at(l, j, k)] = y; });
         });
-        fx_element_max<mm>(st + kFxT1, (unsigned)most.value());
-        if (least < 0 || far > kFxRange || kw > 800 || kw < -800 || kq + kw > 800 || kq + kw < -800) st[kFxLeft1] = 1;
-    }
-    __syncthreads();
+        const int wab = act ? c_fxd[N].wm[a] + c_fxd[N].wm[b] : 0;
+        if (act) fx30_scan<N, 1>(wJ + (e0 + el) * MP + r, {0}, wab, st + kFxW);
+        __syncthreads();
+        for_tasks<m * n, EPB_>(nel, [&](int e, int t) {
+            const long long *Y = boxes + e * C::per + C::SA;
+            long long *X = boxes + e * C::per;
+            const int i = t % m, k = t / m;
+            FxMost most;
+            fx_line<m, n, 1, oI>([&](int l) { return Y[B1::at(i, l, k)]; },
+                                 [&](int l, long long y) {
+                                     X[B2::at(i, l, k)] = y;
+                                     most.see(y);
+                                 });
+            atomicMax(stats + e * K + kFxI, (unsigned)most.value());
+        });
+        __syncthreads();
 
-    // projection along s and r
-    fx30_project_s<N, EPB_, B1, B2>(nel, boxes, boxes + C::SA, C::per, stats, kFxT1);
-    __syncthreads();
-    fx30_project_r<N, EPB_, B1>(
-        nel, boxes + C::SA, C::per, stats, kFxT1, kFxLeft1, [&](int e) { return fx1_exponent<N>(stats + e * K); },
-        [&](int e, int t, int l, double w) { Mq[(e0 + e) * NP + t * n + l] = w; });
-    for (int e = 0; e < nel; e++)
-        if (stats[e * K + kFxLeft1] != 0)  // the same for every thread
-            bp1_element64(reinterpret_cast<double *>(smem_raw), n, oI, oIT, wJ + (e0 + e) * MP, q + (e0 + e) * NP,
-                          Mq + (e0 + e) * NP);
+        // column (a, b): interpolation, wJ and projection along t
+        if (act) {
+            long long *X = boxes + el * C::per, w[m];
+            const int kw = (int)(st[kFxW] >> 20) - 1022, bw = kw + 1022 + wab;
+            int far = 0, least = 0;
+            const double *we = wJ + (e0 + el) * MP + r;
+            const int up = fx30_up<N>(st);
+            fx_line<m, n, 1, oI>([&](int l) { return X[B2::at(a, b, l)] << up; },
+                                 [&](int c, long long g) {
+                                     w[c] = fx30_mass(__ldg(we + c * mm), bw + c_fxd[N].wm[c], g, far, least);
+                                 });
+            FxMost most;
+            fx_apply<n, m, 1, oIT>(w, [&](int l, long long y) {
+                X[B2::at(a, b, l)] = y;
+                most.see(y);
+            });
+            fx_element_max<mm>(st + kFxT1, (unsigned)most.value());
+            if (least < 0 || far > kFxRange || kw > 800 || kw < -800 || kq + kw > 800 || kq + kw < -800)
+                st[kFxLeft1] = flag[1] = 1;
+        }
+        __syncthreads();
+
+        // projection along s and r
+        fx30_project_s<N, EPB_, B1, B2>(nel, boxes, boxes + C::SA, C::per, stats, kFxT1);
+        __syncthreads();
+        fx30_project_r<N, EPB_, B1>(
+            nel, boxes + C::SA, C::per, stats, kFxT1, kFxLeft1, [&](int e) { return fx1_exponent<N>(stats + e * K); },
+            [&](int e, int t, int l, double w) { Mq[(e0 + e) * NP + t * n + l] = w; });
+    }
+    if (flag[1] != 0) bp1_left64<N, EPB_>(smem_raw, e0, nel, wJ, q, Mq);
 }
 
 // ---------------------------------------------------------------- BP3.0
 
 // Shared memory of EPB elements: four m^3 boxes, a word per line, the
-// statistics.
+// statistics, the block's flags (as in Fx1Layout).
 template <int N, int EPB_>
 struct Fx30Layout {
     static constexpr int n = N + 1, m = N + 2, nn = n * n, mm = m * m, NP = nn * n, MP = mm * m, EPB = EPB_;
@@ -444,9 +442,105 @@ struct Fx30Layout {
     static constexpr int threads = ((mm * EPB + 31) / 32) * 32;
     static constexpr int off_e = EPB * per * 8;
     static constexpr int off_s = off_e + EPB * 3 * mm * 4;
-    static constexpr int smem_ = off_s + EPB * kFx30Stats * 4;
+    static constexpr int off_b = off_s + EPB * kFx30Stats * 4;  // the block's flags
+    static constexpr int smem_ = off_b + 8;
     static constexpr int smem = smem_ > threads * 8 ? smem_ : threads * 8;
 };
+
+// Algorithm 5 (MASS: and Algorithm 3) in FP64 on the elements left to it, all at
+// once, in the boxes of the fixed-point path.  Returns the thread's share of q . Aq.
+template <int N, int EPB_, bool MASS>
+__device__ __noinline__ double bp30_left64(unsigned char *smem_raw, int64_t e0, int nel, const double *G, double lambda,
+                                           const double *q, double *Aq, double *Mq) {
+    using C = Fx30Layout<N, EPB_>;
+    using B0 = typename C::B0;
+    using B1 = typename C::B1;
+    using B2 = typename C::B2;
+    using B3 = typename C::B3;
+    constexpr int n = C::n, m = C::m, nn = C::nn, mm = C::mm, NP = C::NP, MP = C::MP, S = C::S, per = C::per;
+    constexpr int oI = fold_offset(N, kFoldI), oIT = fold_offset(N, kFoldIT);
+    constexpr int oDt = fold_offset(N, kFoldDt), oDtT = fold_offset(N, kFoldDtT);
+    const unsigned *stats = reinterpret_cast<const unsigned *>(smem_raw + C::off_s);
+    double *boxes = reinterpret_cast<double *>(smem_raw);
+    auto on30 = [&](int e) { return stats[e * kFx30Stats + kFxLeft30] != 0; };
+    auto on1 = [&](int e) { return MASS && stats[e * kFx30Stats + kFxLeft1] != 0; };
+    auto on = [&](int e) { return on30(e) || on1(e); };
+    const int el = threadIdx.x / mm, r = threadIdx.x - el * mm, u = r % m, v = r / m;
+    const bool act = el < nel && on(el), act30 = el < nel && on30(el);
+    double *A = boxes + el * per, *B = A + S, *Cx = B + S, *D = Cx + S;
+    const double *Ge = G + (e0 + el) * 7 * MP + r;
+    __syncthreads();  // the shared memory is free
+    if (act && r < nn) {
+#pragma unroll
+        for (int k = 0; k < n; k++) B[B0::at(r % n, r / n, k)] = q[(e0 + el) * NP + r + k * nn];
+    }
+    __syncthreads();
+    // interpolation along r (B -> C), s (C -> B) and t (B -> A)
+    fx30_interpolate64<N, EPB_, B0, B1, B2>(nel, boxes + S, boxes + 2 * S, per, on);
+    if (act)
+        fx_from64<m, n, 1, oI>([&](int l) { return B[B2::at(u, v, l)]; }, [&](int l, double y) { A[B3::at(u, v, l)] = y; });
+    __syncthreads();
+    if constexpr (MASS) {  // wJ and projection (A -> B -> C -> Mq)
+        if (act && on1(el))
+            fx_from64<n, m, 1, oIT>([&](int c) { return __dmul_rn(A[B3::at(u, v, c)], __ldg(Ge + 6 * MP + c * mm)); },
+                                    [&](int l, double y) { B[B2::at(u, v, l)] = y; });
+        __syncthreads();
+        fx30_project64<N, EPB_, B1, B2>(nel, boxes + S, boxes + 2 * S, per, on1, [&](int e, int t, int l, double w) {
+            Mq[(e0 + e) * NP + t * n + l] = w;
+        });
+        __syncthreads();
+    }
+    // derivatives along r (A -> B), s (A -> C) and t (A -> D); the directions take
+    // turns in one loop (side by side they spilled)
+    auto line = [&](auto off, int d, const double *from, double *to) {
+        const int step = d == 0 ? 1 : d == 1 ? B3::sj : B3::sk,
+                  at = d == 0 ? B3::at(0, u, v) : d == 1 ? B3::at(u, 0, v) : B3::at(u, v, 0);
+        fx_from64<m, m, -1, off.value>([&](int l) { return from[at + l * step]; },
+                                       [&](int l, double y) { to[at + l * step] = y; });
+    };
+    using Dt = std::integral_constant<int, oDt>;
+    using DtT = std::integral_constant<int, oDtT>;
+    if (act30) {
+#pragma unroll 1
+        for (int d = 0; d < 3; d++) line(Dt(), d, A, B + d * S);
+    }
+    __syncthreads();
+    if (act30) {
+#pragma unroll 2
+        for (int c = 0; c < m; c++) {
+            const int s = B3::at(u, v, c);
+            const double *g = Ge + c * mm, qr = B[s], qs = Cx[s], qt = D[s], g1 = __ldg(g + MP), g2 = __ldg(g + 2 * MP),
+                         g4 = __ldg(g + 4 * MP);
+            B[s] = fx_dot64(__ldg(g), qr, g1, qs, g2, qt);
+            Cx[s] = fx_dot64(g1, qr, __ldg(g + 3 * MP), qs, g4, qt);
+            D[s] = fx_dot64(g2, qr, g4, qs, __ldg(g + 5 * MP), qt);
+        }
+    }
+    __syncthreads();
+    if (act30) {
+#pragma unroll 1
+        for (int d = 0; d < 3; d++) line(DtT(), d, B + d * S, B + d * S);
+    }
+    __syncthreads();
+    // column: the three directions, lambda wJ q and projection along t (D in place), s (D -> C) and r (C -> Aq)
+    if (act30)
+        fx_from64<n, m, 1, oIT>(
+            [&](int c) {
+                const int s = B3::at(u, v, c);
+                double w = D[s];
+                if (lambda != 0.0) w = fma(__dmul_rn(lambda, __ldg(Ge + 6 * MP + c * mm)), A[s], w);
+                return w + (B[s] + Cx[s]);
+            },
+            [&](int l, double y) { D[B2::at(u, v, l)] = y; });
+    __syncthreads();
+    double dot = 0.0;
+    fx30_project64<N, EPB_, B1, B2>(nel, boxes + 3 * S, boxes + 2 * S, per, on30, [&](int e, int t, int l, double w) {
+        const int64_t g = (e0 + e) * NP + t * n + l;
+        Aq[g] = w;
+        dot = fma(q[g], w, dot);
+    });
+    return dot;
+}
 
 // BP3.0 of elements [e0, e0 + nel) by the whole block (blockDim.x >=
 // Layout::threads); MASS: BP1.0 too, to Mq, with wJ the seventh factor.  PCG
@@ -473,11 +567,14 @@ __device__ __forceinline__ void bp30_fx_block(unsigned char *smem_raw, int64_t e
     int *ln = reinterpret_cast<int *>(smem_raw + C::off_e) + el * 3 * mm;
     unsigned *stats = reinterpret_cast<unsigned *>(smem_raw + C::off_s), *st = stats + el * K;
     if (threadIdx.x == 0) prefetch_l2(G + e0 * 7 * MP, (long long)nel * 7 * MP * 8);
-    for (int t = threadIdx.x; t < EPB_ * K; t += blockDim.x) stats[t] = 0;
+    volatile unsigned *flag = reinterpret_cast<volatile unsigned *>(smem_raw + C::off_b);
+    for (int t = threadIdx.x; t < EPB_ * K + 2; t += blockDim.x) stats[t] = 0;  // (the flags lie behind them)
     __syncthreads();
 
     double qv[n];
     const bool col = act && r < nn;
+    const double *Ge = G + (e0 + el) * 7 * MP + r;
+    const int sign = act ? fx30_sign(Ge) : 0, sign1 = MASS && act ? fx30_sign(Ge + 6 * MP) : 0;
     if (col) fx30_load<N, PCG>(qv, (e0 + el) * NP + r, r, q, z, p, beta, st);
     __syncthreads();
     int kq = 0;
@@ -492,203 +589,194 @@ __device__ __forceinline__ void bp30_fx_block(unsigned char *smem_raw, int64_t e
                 B[B0::at(r % n, r / n, k)] = fx_from_double<qb>(qv[k], kq + 1022 - e);
             }
         }
-        if (left) st[kFxLeft1] = st[kFxLeft30] = 1;
+        if (left || sign1 < 0) st[kFxLeft1] = 1;
+        if (left || sign < 0) st[kFxLeft30] = 1;
+        if (left || sign < 0 || sign1 < 0) flag[1] = 1;
+        if (!left && (sign >= 0 || (MASS && sign1 >= 0))) flag[0] = 1;
     }
-    __syncthreads();
-
-    // interpolation along r (B -> C), s (C -> B) and t (B -> A)
-    for_tasks<nn, EPB_>(nel, [&](int e, int t) {
-        const long long *X = boxes + e * C::per + S;
-        long long *Y = boxes + e * C::per + 2 * S;
-        const int j = t % n, k = t / n;
-        fx_line<m, n, 1, oI>([&](int l) { return X[B0::at(l, j, k)]; }, [&](int l, long long y) { Y[B1::at(l, j, k)] = y; });
-    });
-    __syncthreads();
-    for_tasks<m * n, EPB_>(nel, [&](int e, int t) {
-        const long long *Y = boxes + e * C::per + 2 * S;
-        long long *X = boxes + e * C::per + S;
-        const int i = t % m, k = t / m;
-        FxMost most;
-        fx_line<m, n, 1, oI>([&](int l) { return Y[B1::at(i, l, k)]; },
-                             [&](int l, long long y) {
-                                 X[B2::at(i, l, k)] = y;
-                                 most.see(y);
-                             });
-        atomicMax(stats + e * K + kFxI, (unsigned)most.value());
-    });
-    __syncthreads();
-    const double *Ge = G + (e0 + el) * 7 * MP + r;
-    const int wuv = act ? c_fxd[N].wm[u] + c_fxd[N].wm[v] : 0;
-    int t3 = 3 * c_fxd[N].tau[kFoldI];  // exponent of the interpolated field over q's
-    if (act) {
-        t3 -= fx30_up<N>(st);
-        const int up = fx30_up<N>(st);
-        fx_line<m, n, 1, oI>([&](int l) { return B[B2::at(u, v, l)] << up; },
-                             [&](int l, long long y) { A[B3::at(u, v, l)] = y; });
-        fx30_scan<N, 4>(Ge, {6, 0, 3, 5}, wuv, st + kFxW);
-    }
-    __syncthreads();
-    const int kw = act ? (int)(st[kFxW] >> 20) - 1022 : 0;
-
-    // BP1.0: wJ and projection along t (A -> B), s (B -> C) and r (C -> Mq)
-    if constexpr (MASS) {
-        if (act) {
-            long long w[m];
-            const int bw = kw + 1022 + wuv;
-            int far = 0, least = 0;
-#pragma unroll
-            for (int c = 0; c < m; c++)
-                w[c] = fx30_mass(__ldg(Ge + 6 * MP + c * mm), bw + c_fxd[N].wm[c], A[B3::at(u, v, c)], far, least);
-            FxMost most;
-            fx_apply<n, m, 1, oIT>(w, [&](int l, long long y) {
-                B[B2::at(u, v, l)] = y;
-                most.see(y);
-            });
-            fx_element_max<mm>(st + kFxT1, (unsigned)most.value());
-            if (least < 0 || far > kFxRange || kw > 800 || kw < -800 || kq + kw > 800 || kq + kw < -800)
-                st[kFxLeft1] = 1;
-        }
-        __syncthreads();
-        fx30_project_s<N, EPB_, B1, B2>(nel, boxes + S, boxes + 2 * S, C::per, stats, kFxT1);
-        __syncthreads();
-        fx30_project_r<N, EPB_, B1>(
-            nel, boxes + 2 * S, C::per, stats, kFxT1, kFxLeft1, [&](int e) { return fx1_exponent<N>(stats + e * K); },
-            [&](int e, int t, int l, double w) { Mq[(e0 + e) * NP + t * n + l] = w; });
-        __syncthreads();
-    }
-
-    // derivatives along r (A -> B), s (A -> C) and t (A -> D)
-    if (act) {
-        const int mr = fx_derivative<B3, m, oDt, 0>(A, B, u, v), ms = fx_derivative<B3, m, oDt, 1>(A, Cx, u, v),
-                  mt = fx_derivative<B3, m, oDt, 2>(A, D, u, v);
-        fx_element_max<mm>(st + kFxU, (unsigned)mr);
-        fx_element_max<mm>(st + kFxU + 1, (unsigned)ms);
-        fx_element_max<mm>(st + kFxU + 2, (unsigned)mt);
-    }
-    __syncthreads();
-
-    // chain rule at the points of column (a=u, b=v)
-    int basez = 0;
-    if (act) {
-        const FxScales<QB> Z(st + kFxG);
-        const int kg = Z.kg;
-        const bool left = Z.bad || kq + kg > 800 || kq + kg < -800;
-        basez = kq - qb + t3 + c_fxd[N].tau[kFoldDt] - Z.sh + 2 + kg + c_fxd[N].tau[kFoldDtT];
-        const int eg = kg + 1022 + wuv;
-        FxRange range;
-        auto chain = [&](int c, auto split) {
-            const int s = B3::at(u, v, c);
-            fx_chain<split.value>(Ge + c * mm, MP, eg + c_fxd[N].wm[c], Z, B[s], Cx[s], D[s], B[s], Cx[s], D[s], range);
-        };
-        if (!Z.split) {
-#pragma unroll 4
-            for (int c = 0; c < m; c++) chain(c, std::false_type());
-        } else {
-#pragma unroll 1
-            for (int c = 0; c < m; c++) chain(c, std::true_type());
-        }
-        if (left || range.left()) st[kFxLeft30] = 1;
-        if (r == 0) st[kFxB] = Z.below();
-    }
-    __syncthreads();
-
-    // transposes, in place; ln: each line's scale
-    if (act) {
-        const unsigned below = st[kFxB];
-        const int hr = fx_transpose<B3, m, oDtT, QB, 0, EXACT>(B, u, v) + fx_below(below, 0),
-                  hs = fx_transpose<B3, m, oDtT, QB, 1, EXACT>(Cx, u, v) + fx_below(below, 1),
-                  ht = fx_transpose<B3, m, oDtT, QB, 2, EXACT>(D, u, v) + fx_below(below, 2);
-        ln[r] = hr;
-        ln[mm + r] = hs;
-        ln[2 * mm + r] = ht;
-        const int h = __vimin3_s32(hr, hs, ht);
-        if (!EXACT || h < kFxZeroLine) fx_element_max<EXACT ? 1 : mm>(st + kFxH, (unsigned)(63 - h));
-        if (EXACT) {
-            const int unit = __vimin3_s32(hr < kFxZeroLine ? fx_below(below, 0) : 63, hs < kFxZeroLine ? fx_below(below, 1) : 63,
-                                          ht < kFxZeroLine ? fx_below(below, 2) : 63);
-            atomicMax(st + kFxE, (unsigned)(63 - unit));
-        }
-    }
-    __syncthreads();
-
-    // column: the three directions and lambda wJ q, aligned (-> D)
-    int zs = 0;
-    if (act) {
-        // every line is brought to the largest scale among them (N = 1: that are not zero)
-        const int hm = (EXACT && st[kFxH] == 0) ? QB - 32 : 63 - (int)st[kFxH];
-        basez -= hm;
-        // lines are known to a unit of their direction's scale: the largest
-        // must not lie far below that of the largest that is not zero
-        const bool lost = EXACT && st[kFxH] != 0 && st[kFxH] + kFxRange < st[kFxE];
-        int el2 = 0;  // |lambda| < 2^el2
-        if (lambda != 0.0) el2 = ((__double2hiint(lambda) >> 20) & 0x7ff) - 1022;
-        const int delta = kq - qb + t3 + kw + el2 - basez;  // scale of the mass term over the other's
-        zs = (lambda != 0.0) ? min(63, max(0, delta)) : 0;
-        const int ms = min(63, max(0, -delta)), bw = kw + el2 + 1022 + wuv, ht = ln[2 * mm + r] - hm + zs;
-        bool left = el2 > 200 || el2 < -200 || delta > 63 || kw > 800 || kw < -800 || kq + kw > 800 || kq + kw < -800;
-        if (lambda == 0.0) left = false;
-        left = left || lost;
-        FxMost most;
-        int far = 0, least = 0;
-#pragma unroll 4
-        for (int c = 0; c < m; c++) {
-            const int s = B3::at(u, v, c);
-            long long x = fx_shr(B[s], ln[v + m * c] - hm + zs) + fx_shr(Cx[s], ln[mm + u + m * c] - hm + zs) +
-                          fx_shr(D[s], ht);
-            if (lambda != 0.0) {
-                const double wj = lambda * __ldg(Ge + 6 * MP + c * mm);
-                const int e = (__double2hiint(wj) >> 20) & 0x7ff, d = bw + c_fxd[N].wm[c] - e;
-                far = max(far, d);
-                least = min(least, d);
-                int gh, gl;
-                fx_off_diagonal(wj, d, gh, gl);
-                x += fx_mul(gh, gl, A[s]) >> ms;
-            }
-            D[s] = x;
-            most.see(x);
-        }
-        fx_element_max<mm>(st + kFxX, (unsigned)most.value());
-        if (left || least < 0 || far > kFxRange + 2) st[kFxLeft30] = 1;
-    }
-    __syncthreads();
-
-    // projection along t (D in place), s (D -> C) and r (C -> Aq)
-    if (act) {
-        const int sx = QB - 32 - fx_top((int)st[kFxX]), up = max(0, sx), down = max(0, -sx);
-        FxMost most;
-        fx_line<n, m, 1, oIT>([&](int l) { return (D[B3::at(u, v, l)] << up) >> down; },
-                              [&](int l, long long y) {
-                                  D[B2::at(u, v, l)] = y;
-                                  most.see(y);
-                              });
-        fx_element_max<mm>(st + kFxT30, (unsigned)most.value());
-        if (r == 0) ln[0] = basez + zs - sx + 3 * c_fxd[N].tau[kFoldIT];  // (every line's scale has been read)
-    }
-    __syncthreads();
-    fx30_project_s<N, EPB_, B1, B2>(nel, boxes + 3 * S, boxes + 2 * S, C::per, stats, kFxT30);
     __syncthreads();
     double dot = 0.0;  // p . Ap of the thread's lines
-    fx30_project_r<N, EPB_, B1>(
-        nel, boxes + 2 * S, C::per, stats, kFxT30, kFxLeft30,
-        [&](int e) { return reinterpret_cast<const int *>(smem_raw + C::off_e)[e * 3 * mm]; },
-        [&](int e, int t, int l, double w) {
-            const int64_t g = (e0 + e) * NP + t * n + l;
-            Aq[g] = w;
-            if (PCG) dot = fma(p[g], w, dot);
+    if (flag[0] != 0) {
+        // interpolation along r (B -> C), s (C -> B) and t (B -> A)
+        for_tasks<nn, EPB_>(nel, [&](int e, int t) {
+            const long long *X = boxes + e * C::per + S;
+            long long *Y = boxes + e * C::per + 2 * S;
+            const int j = t % n, k = t / n;
+            fx_line<m, n, 1, oI>([&](int l) { return X[B0::at(l, j, k)]; }, [&](int l, long long y) { Y[B1::at(l, j, k)] = y; });
         });
-    for (int e = 0; e < nel; e++) {  // (the conditions are the same for every thread)
-        const int64_t g0 = (e0 + e) * NP;
-        const double *qe = (PCG ? p : q) + g0, *ge = G + (e0 + e) * 7 * MP;
-        if (MASS && stats[e * K + kFxLeft1] != 0)
-            bp1_element64(reinterpret_cast<double *>(smem_raw), n, oI, oIT, ge + 6 * MP, qe, Mq + g0);
-        if (stats[e * K + kFxLeft30] != 0) {
-            bp30_element64(reinterpret_cast<double *>(smem_raw), n, oI, oIT, oDt, oDtT, ge, lambda, qe, Aq + g0);
-            if (PCG) {
-                __syncthreads();  // (the element's output is there)
-                for (int t = threadIdx.x; t < NP; t += blockDim.x) dot = fma(qe[t], Aq[g0 + t], dot);
+        __syncthreads();
+        for_tasks<m * n, EPB_>(nel, [&](int e, int t) {
+            const long long *Y = boxes + e * C::per + 2 * S;
+            long long *X = boxes + e * C::per + S;
+            const int i = t % m, k = t / m;
+            FxMost most;
+            fx_line<m, n, 1, oI>([&](int l) { return Y[B1::at(i, l, k)]; },
+                                 [&](int l, long long y) {
+                                     X[B2::at(i, l, k)] = y;
+                                     most.see(y);
+                                 });
+            atomicMax(stats + e * K + kFxI, (unsigned)most.value());
+        });
+        __syncthreads();
+        const int wuv = act ? c_fxd[N].wm[u] + c_fxd[N].wm[v] : 0;
+        int t3 = 3 * c_fxd[N].tau[kFoldI];  // exponent of the interpolated field over q's
+        if (act) {
+            t3 -= fx30_up<N>(st);
+            const int up = fx30_up<N>(st);
+            fx_line<m, n, 1, oI>([&](int l) { return B[B2::at(u, v, l)] << up; },
+                                 [&](int l, long long y) { A[B3::at(u, v, l)] = y; });
+            fx30_scan<N, 4>(Ge, {6, 0, 3, 5}, wuv, st + kFxW);
+        }
+        __syncthreads();
+        const int kw = act ? (int)(st[kFxW] >> 20) - 1022 : 0;
+
+        // BP1.0: wJ and projection along t (A -> B), s (B -> C) and r (C -> Mq)
+        if constexpr (MASS) {
+            if (act) {
+                long long w[m];
+                const int bw = kw + 1022 + wuv;
+                int far = 0, least = 0;
+#pragma unroll
+                for (int c = 0; c < m; c++)
+                    w[c] = fx30_mass(__ldg(Ge + 6 * MP + c * mm), bw + c_fxd[N].wm[c], A[B3::at(u, v, c)], far, least);
+                FxMost most;
+                fx_apply<n, m, 1, oIT>(w, [&](int l, long long y) {
+                    B[B2::at(u, v, l)] = y;
+                    most.see(y);
+                });
+                fx_element_max<mm>(st + kFxT1, (unsigned)most.value());
+                if (least < 0 || far > kFxRange || kw > 800 || kw < -800 || kq + kw > 800 || kq + kw < -800)
+                    st[kFxLeft1] = flag[1] = 1;
+            }
+            __syncthreads();
+            fx30_project_s<N, EPB_, B1, B2>(nel, boxes + S, boxes + 2 * S, C::per, stats, kFxT1);
+            __syncthreads();
+            fx30_project_r<N, EPB_, B1>(
+                nel, boxes + 2 * S, C::per, stats, kFxT1, kFxLeft1, [&](int e) { return fx1_exponent<N>(stats + e * K); },
+                [&](int e, int t, int l, double w) { Mq[(e0 + e) * NP + t * n + l] = w; });
+            __syncthreads();
+        }
+
+        // derivatives along r (A -> B), s (A -> C) and t (A -> D)
+        if (act) {
+            const int mr = fx_derivative<B3, m, oDt, 0>(A, B, u, v), ms = fx_derivative<B3, m, oDt, 1>(A, Cx, u, v),
+                      mt = fx_derivative<B3, m, oDt, 2>(A, D, u, v);
+            fx_element_max<mm>(st + kFxU, (unsigned)mr);
+            fx_element_max<mm>(st + kFxU + 1, (unsigned)ms);
+            fx_element_max<mm>(st + kFxU + 2, (unsigned)mt);
+        }
+        __syncthreads();
+
+        // chain rule at the points of column (a=u, b=v)
+        int basez = 0;
+        if (act) {
+            const FxScales<QB> Z(st + kFxG);
+            const int kg = Z.kg;
+            const bool left = Z.bad || kq + kg > 800 || kq + kg < -800;
+            basez = kq - qb + t3 + c_fxd[N].tau[kFoldDt] - Z.sh + 2 + kg + c_fxd[N].tau[kFoldDtT];
+            const int eg = kg + 1022 + wuv;
+            FxRange range;
+            auto chain = [&](int c, auto split) {
+                const int s = B3::at(u, v, c);
+                fx_chain<split.value>(Ge + c * mm, MP, eg + c_fxd[N].wm[c], Z, B[s], Cx[s], D[s], B[s], Cx[s], D[s], range);
+            };
+            if (!Z.split) {
+#pragma unroll 4
+                for (int c = 0; c < m; c++) chain(c, std::false_type());
+            } else {
+#pragma unroll 1
+                for (int c = 0; c < m; c++) chain(c, std::true_type());
+            }
+            if (left || range.left()) st[kFxLeft30] = flag[1] = 1;
+            if (r == 0) st[kFxB] = Z.below();
+        }
+        __syncthreads();
+
+        // transposes, in place; ln: each line's scale
+        if (act) {
+            const unsigned below = st[kFxB];
+            const int hr = fx_transpose<B3, m, oDtT, QB, 0, EXACT>(B, u, v) + fx_below(below, 0),
+                      hs = fx_transpose<B3, m, oDtT, QB, 1, EXACT>(Cx, u, v) + fx_below(below, 1),
+                      ht = fx_transpose<B3, m, oDtT, QB, 2, EXACT>(D, u, v) + fx_below(below, 2);
+            ln[r] = hr;
+            ln[mm + r] = hs;
+            ln[2 * mm + r] = ht;
+            const int h = __vimin3_s32(hr, hs, ht);
+            if (!EXACT || h < kFxZeroLine) fx_element_max<EXACT ? 1 : mm>(st + kFxH, (unsigned)(63 - h));
+            if (EXACT) {
+                const int unit = __vimin3_s32(hr < kFxZeroLine ? fx_below(below, 0) : 63, hs < kFxZeroLine ? fx_below(below, 1) : 63,
+                                              ht < kFxZeroLine ? fx_below(below, 2) : 63);
+                atomicMax(st + kFxE, (unsigned)(63 - unit));
             }
         }
+        __syncthreads();
+
+        // column: the three directions and lambda wJ q, aligned (-> D)
+        int zs = 0;
+        if (act) {
+            // every line is brought to the largest scale among them (N = 1: that are not zero)
+            const int hm = (EXACT && st[kFxH] == 0) ? QB - 32 : 63 - (int)st[kFxH];
+            basez -= hm;
+            // lines are known to a unit of their direction's scale: the largest
+            // must not lie far below that of the largest that is not zero
+            const bool lost = EXACT && st[kFxH] != 0 && st[kFxH] + kFxRange < st[kFxE];
+            int el2 = 0;  // |lambda| < 2^el2
+            if (lambda != 0.0) el2 = ((__double2hiint(lambda) >> 20) & 0x7ff) - 1022;
+            const int delta = kq - qb + t3 + kw + el2 - basez;  // scale of the mass term over the other's
+            zs = (lambda != 0.0) ? min(63, max(0, delta)) : 0;
+            const int ms = min(63, max(0, -delta)), bw = kw + el2 + 1022 + wuv, ht = ln[2 * mm + r] - hm + zs;
+            bool left = el2 > 200 || el2 < -200 || delta > 63 || kw > 800 || kw < -800 || kq + kw > 800 || kq + kw < -800;
+            if (lambda == 0.0) left = false;
+            left = left || lost;
+            FxMost most;
+            int far = 0, least = 0;
+#pragma unroll 4
+            for (int c = 0; c < m; c++) {
+                const int s = B3::at(u, v, c);
+                long long x = fx_shr(B[s], ln[v + m * c] - hm + zs) + fx_shr(Cx[s], ln[mm + u + m * c] - hm + zs) +
+                              fx_shr(D[s], ht);
+                if (lambda != 0.0) {
+                    const double wj = lambda * __ldg(Ge + 6 * MP + c * mm);
+                    const int e = (__double2hiint(wj) >> 20) & 0x7ff, d = bw + c_fxd[N].wm[c] - e;
+                    far = max(far, d);
+                    least = min(least, d);
+                    int gh, gl;
+                    fx_off_diagonal(wj, d, gh, gl);
+                    x += fx_mul(gh, gl, A[s]) >> ms;
+                }
+                D[s] = x;
+                most.see(x);
+            }
+            fx_element_max<mm>(st + kFxX, (unsigned)most.value());
+            if (left || least < 0 || far > kFxRange + 2) st[kFxLeft30] = flag[1] = 1;
+        }
+        __syncthreads();
+
+        // projection along t (D in place), s (D -> C) and r (C -> Aq)
+        if (act) {
+            const int sx = QB - 32 - fx_top((int)st[kFxX]), up = max(0, sx), down = max(0, -sx);
+            FxMost most;
+            fx_line<n, m, 1, oIT>([&](int l) { return (D[B3::at(u, v, l)] << up) >> down; },
+                                  [&](int l, long long y) {
+                                      D[B2::at(u, v, l)] = y;
+                                      most.see(y);
+                                  });
+            fx_element_max<mm>(st + kFxT30, (unsigned)most.value());
+            if (r == 0) ln[0] = basez + zs - sx + 3 * c_fxd[N].tau[kFoldIT];  // (every line's scale has been read)
+        }
+        __syncthreads();
+        fx30_project_s<N, EPB_, B1, B2>(nel, boxes + 3 * S, boxes + 2 * S, C::per, stats, kFxT30);
+        __syncthreads();
+        fx30_project_r<N, EPB_, B1>(
+            nel, boxes + 2 * S, C::per, stats, kFxT30, kFxLeft30,
+            [&](int e) { return reinterpret_cast<const int *>(smem_raw + C::off_e)[e * 3 * mm]; },
+            [&](int e, int t, int l, double w) {
+                const int64_t g = (e0 + e) * NP + t * n + l;
+                Aq[g] = w;
+                if (PCG) dot = fma(p[g], w, dot);
+            });
     }
+    if (flag[1] != 0) dot += bp30_left64<N, EPB_, MASS>(smem_raw, e0, nel, G, lambda, PCG ? p : q, Aq, Mq);
     if (PCG) {
         __syncthreads();  // the shared boxes are reused for the reduction
         const double tot = block_sum(dot, reinterpret_cast<double *>(smem_raw));

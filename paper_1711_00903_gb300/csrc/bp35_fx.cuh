@@ -24,14 +24,11 @@
 // 0.9) and 0.2 to 0.8 for smooth ones.
 //
 // An element whose values do not share a scale is computed in FP64 instead
-// (bp35_element64), by the same block: non-finite or extreme values,
+// (bp35_lines64), by the same block: non-finite or extreme values,
 // a node whose result is made of values all far smaller than the element's
 // largest (in FP64 it keeps digits that the element's scale cuts off), a
 // point whose factors are far smaller than the element's largest, or an
-// off-diagonal factor above every diagonal one (G not positive definite).  At
-// two and three points a line, where FP64 takes the derivative of a constant
-// (at two of any line) without an error, also a node whose lines hold far less
-// than the scale of the directions that reach it.
+// off-diagonal factor above every diagonal one (G not positive definite).
 // The choice is made element by element, so a result does not depend on the
 // other elements of the block.  Of a smooth field that vanishes on the faces
 // of a box, the elements along the box's edges go this way (0.6 % of 32^3
@@ -45,65 +42,115 @@
 namespace fem {
 namespace {
 
+// Slots of an element's statistics: the largest q, Grr, Gss, Gtt and
+// derivatives along r, s, t (FxScales), whether the element is left to FP64,
+// whether it holds values below a unit, the directions' scales (fx_below), the
+// largest q of each face.
+enum { kFx35Q = 0, kFx35G = 1, kFx35Left = 7, kFx35Tiny = 8, kFx35B = 9, kFx35F = 10, kFx35Stats = 16 };
+
+// At two and three points a line BP3.5 stays in FP64: its derivatives of a
+// constant line (at two points of any line) have no error there, so a node far
+// below its element's largest keeps digits that one scale cuts off, and of a
+// smooth field so many elements hold such nodes that the fixed point gained
+// nothing (N = 1, 2 on a product of sines: 46 and 78 us against 40 and 78).
+__host__ __device__ constexpr bool fx35_fixed(int N) { return N >= 3; }
+
 template <int N, int EPB_>
 struct Fx35Layout : Bp35Layout<double, N, EPB_> {
     using L = Bp35Layout<double, N, EPB_>;
-    // per element: max q; max Grr, Gss, Gtt; max derivative along r, s, t; left out; values below a unit;
-    // the directions' scales (fx_below)
-    static constexpr int kStats = 10;
-    // boxes, then a word per line, then the statistics
+    static constexpr int kStats = kFx35Stats;
+    // boxes, then a word per line, the statistics and three flags of the block: an
+    // element is on the fixed-point path; one is left to FP64; one has a small corner
     static constexpr int off_e = L::bytes;
     static constexpr int off_s = off_e + EPB_ * 3 * L::nn * 4;
-    static constexpr int fx_bytes = off_s + EPB_ * kStats * 4;
+    static constexpr int off_b = off_s + EPB_ * kStats * 4;  // the block's flags
+    static constexpr int fx_bytes = off_b + 12;
     static constexpr int smem = fx_bytes > L::smem ? fx_bytes : L::smem;
 };
 
-// Algorithm 4 in FP64 on one element by the whole block, sizes at run time
-// (fx_line64): q, G and Aq at the element, smem at least 3 n^3 doubles (rows
-// of n, or n + 1 for even n, against bank conflicts).  Returns the thread's
-// share of q . Aq.
-__device__ __noinline__ double bp35_element64(double *smem, int n, int oD, int oDT, const double *G, double lambda,
-                                              const double *q, double *Aq) {
-    const int nn = n * n, NP = nn * n, sj = n | 1, sk = sj * n, size = sk * n;
-    double *sQ = smem, *sR = sQ + size, *sS = sR + size;
+// Algorithm 4 in FP64 on the block's elements [e0, e0 + nel) for which on(el)
+// holds, all of them at once, a line per thread as on the fixed-point path and
+// in its boxes.  Returns the thread's share of q . Aq.
+template <int N, int EPB_, class F>
+__device__ __forceinline__ double bp35_lines64(unsigned char *smem_raw, int64_t e0, int nel, const double *G,
+                                               double lambda, const double *q, double *Aq, F &&on) {
+    using C = Fx35Layout<N, EPB_>;
+    using B = typename C::B;
+    constexpr int n = C::n, nn = C::nn, NP = C::NP;
+    constexpr int oD = fold_offset(N, kFoldD), oDT = fold_offset(N, kFoldDT);
+    const int el = threadIdx.x / nn, r = threadIdx.x - el * nn;
+    const int u = r % n, v = r / n;
+    const bool act = el < nel && on(el);
+    const int64_t g0 = (e0 + el) * NP + r;
+    double *box = reinterpret_cast<double *>(smem_raw) + el * 3 * B::size, *bs = box + B::size, *bt = bs + B::size;
+    // the thread's line of direction d from one box to another, or in place; the
+    // directions take turns in one loop (side by side they spilled)
+    auto line = [&](auto off, int d, const double *from, double *to) {
+        const int step = d == 0 ? 1 : d == 1 ? B::sj : B::sk,
+                  at = d == 0 ? B::at(0, u, v) : d == 1 ? B::at(u, 0, v) : B::at(u, v, 0);
+        double x[n];
+#pragma unroll
+        for (int l = 0; l < n; l++) x[l] = from[at + l * step];
+        fx_line64<n, n, -1, off.value>(x, [&](int l, double y) { to[at + l * step] = y; });
+    };
+    using D = std::integral_constant<int, oD>;
+    using DT = std::integral_constant<int, oDT>;
     __syncthreads();  // the shared memory is free
-    for (int t = threadIdx.x; t < NP; t += blockDim.x) sQ[t % n + sj * ((t / n) % n) + sk * (t / nn)] = q[t];
-    __syncthreads();
-    const int r = threadIdx.x, u = r % n, v = r / n;
-    double ut[kMaxN + 1], acc[kMaxN + 1], dot = 0.0;
-    if (r < nn) {
-        fx_line64(sQ + sj * u + sk * v, 1, sR + sj * u + sk * v, 1, n, n, -1, oD);
-        fx_line64(sQ + u + sk * v, sj, sS + u + sk * v, sj, n, n, -1, oD);
-        fx_line64(sQ + u + sj * v, sk, ut, 1, n, n, -1, oD);
+    if (act) {
+#pragma unroll
+        for (int k = 0; k < n; k++) box[B::at(u, v, k)] = q[g0 + k * nn];
     }
     __syncthreads();
-    if (r < nn) {
-        for (int k = 0; k < n; k++) {
-            const int s = u + sj * v + sk * k;
-            const double *g = G + r + k * nn, qr = sR[s], qs = sS[s], qt = ut[k];
-            sR[s] = g[0] * qr + g[NP] * qs + g[2 * NP] * qt;
-            sS[s] = g[NP] * qr + g[3 * NP] * qs + g[4 * NP] * qt;
-            ut[k] = g[2 * NP] * qr + g[4 * NP] * qs + g[5 * NP] * qt;
+    // derivatives along t and s to boxes 2 and 1, then along r in place in box 0
+#pragma unroll 1
+    for (int d = 2; d >= 0; d--) {
+        if (d == 0) __syncthreads();
+        if (act) line(D(), d, box, box + d * B::size);
+    }
+    __syncthreads();
+    if (act) {
+        const double *g = G + (e0 + el) * 7 * NP + r;
+#pragma unroll 2
+        for (int k = 0; k < n; k++, g += nn) {
+            const int s = B::at(u, v, k);
+            const double qr = box[s], qs = bs[s], qt = bt[s], g1 = __ldg(g + NP), g2 = __ldg(g + 2 * NP),
+                         g4 = __ldg(g + 4 * NP);
+            box[s] = fx_dot64(__ldg(g), qr, g1, qs, g2, qt);
+            bs[s] = fx_dot64(g1, qr, __ldg(g + 3 * NP), qs, g4, qt);
+            bt[s] = fx_dot64(g2, qr, g4, qs, __ldg(g + 5 * NP), qt);
         }
-        fx_line64(ut, 1, acc, 1, n, n, -1, oDT);
     }
     __syncthreads();
-    if (r < nn) {
-        fx_line64(sR + sj * u + sk * v, 1, sR + sj * u + sk * v, 1, n, n, -1, oDT);
-        fx_line64(sS + u + sk * v, sj, sS + u + sk * v, sj, n, n, -1, oDT);
+    if (act) {
+#pragma unroll 1
+        for (int d = 0; d < 3; d++) line(DT(), d, box + d * B::size, box + d * B::size);
     }
     __syncthreads();
-    if (r < nn) {
+    double dot = 0.0;
+    if (act) {
+#pragma unroll 2
         for (int k = 0; k < n; k++) {
-            const int s = u + sj * v + sk * k;
-            double w = acc[k];
-            if (lambda != 0.0) w = fma(lambda, G[6 * NP + r + k * nn] * sQ[s], w);
-            w = w + sR[s] + sS[s];
-            Aq[r + k * nn] = w;
-            dot = fma(sQ[s], w, dot);
+            const int s = B::at(u, v, k);
+            const double qk = q[g0 + k * nn];
+            double w = bt[s];
+            if (lambda != 0.0) w = fma(lambda, __dmul_rn(__ldg(G + (e0 + el) * 7 * NP + 6 * NP + r + k * nn), qk), w);
+            w = w + box[s] + bs[s];
+            Aq[g0 + k * nn] = w;
+            dot = fma(qk, w, dot);
         }
     }
     return dot;
+}
+
+// The same as a function of its own, for the elements that the fixed-point path
+// leaves out (stats: their flags), so that its registers are not the fast path's.
+template <int N, int EPB_>
+__device__ __noinline__ double bp35_left64(unsigned char *smem_raw, int64_t e0, int nel, const double *G, double lambda,
+                                           const double *q, double *Aq) {
+    using C = Fx35Layout<N, EPB_>;
+    const unsigned *stats = reinterpret_cast<const unsigned *>(smem_raw + C::off_s);
+    return bp35_lines64<N, EPB_>(smem_raw, e0, nel, G, lambda, q, Aq,
+                                 [&](int el) { return stats[el * C::kStats + kFx35Left] != 0; });
 }
 
 // Whether node (i, j, k), none of whose lines reaches the element's scale, is
@@ -132,6 +179,48 @@ __device__ __noinline__ bool fx35_held(const int *ln, const double *G, int n, in
     return !any;
 }
 
+// Leaves out elements with a corner whose three faces hold values far below the
+// element's largest only: it is not held to the element's scale (fx35_held reads
+// its faces), which this tells before the contractions, from the scaled field.
+// (Fields that decay across an element are made of such elements.)  Returns
+// whether elements are left on the fixed-point path.
+template <int N, int EPB_>
+__device__ __noinline__ bool fx35_corners(unsigned char *smem_raw, int nel) {
+    using C = Fx35Layout<N, EPB_>;
+    using B = typename C::B;
+    constexpr int n = C::n, nn = C::nn, need = fx_bits35(N) - 1 - 32 - kFxRange;
+    const int el = threadIdx.x / nn, r = threadIdx.x - el * nn, u = r % n, v = r / n;
+    unsigned *stats = reinterpret_cast<unsigned *>(smem_raw + C::off_s), *st = stats + el * C::kStats;
+    if (el < nel) {
+        const long long *box = reinterpret_cast<const long long *>(smem_raw) + el * 3 * B::size;
+        auto value = [&](int k) {
+            const int h = (int)(box[B::at(u, v, k)] >> 32);
+            return (unsigned)max(h, ~h);
+        };
+        unsigned m = 0;
+        for (int k = 0; k < n; k++) m = max(m, value(k));
+        if (u == 0) atomicMax(st + kFx35F, m);
+        if (u == n - 1) atomicMax(st + kFx35F + 1, m);
+        if (v == 0) atomicMax(st + kFx35F + 2, m);
+        if (v == n - 1) atomicMax(st + kFx35F + 3, m);
+        atomicMax(st + kFx35F + 4, value(0));
+        atomicMax(st + kFx35F + 5, value(n - 1));
+    }
+    __syncthreads();
+    if (el < nel && r == 0) {
+        const unsigned *f = st + kFx35F;
+        const unsigned least = max(max(min(f[0], f[1]), min(f[2], f[3])), min(f[4], f[5]));
+        if (least != 0 && fx_top((int)least) < need) {
+            st[kFx35Left] = 1;
+            reinterpret_cast<volatile unsigned *>(smem_raw + C::off_b)[1] = 1;
+        }
+    }
+    __syncthreads();
+    bool some = false;
+    for (int e = 0; e < nel; e++) some = some || stats[e * C::kStats + kFx35Left] == 0;
+    return some;
+}
+
 // BP3.5 of elements [e0, e0 + nel) by the whole block (blockDim.x >=
 // Layout::threads), as bp35_block.
 template <int N, int EPB_, bool PCG>
@@ -142,7 +231,6 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
     using C = Fx35Layout<N, EPB_>;
     using B = typename C::B;
     constexpr int n = C::n, nn = C::nn, NP = C::NP, QB = fx_bits35(N), K = C::kStats;
-    constexpr bool EXACT = n <= 3;  // FP64 lines may make no error
     constexpr int UC = 4;  // nodes of a column taken at a time (whole columns spill)
     constexpr int oD = fold_offset(N, kFoldD), oDT = fold_offset(N, kFoldDT);
     const int el = threadIdx.x / nn, r = threadIdx.x - el * nn;
@@ -152,15 +240,36 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
     int *ln = reinterpret_cast<int *>(smem_raw + C::off_e) + el * 3 * nn;         // a word per line
     unsigned *stats = reinterpret_cast<unsigned *>(smem_raw + C::off_s), *st = stats + el * K;
     if (threadIdx.x == 0) prefetch_l2(G + e0 * 7 * NP, (long long)nel * 7 * NP * 8);
-    for (int t = threadIdx.x; t < EPB_ * K; t += blockDim.x) stats[t] = 0;
+    if constexpr (!fx35_fixed(N)) {
+        if (PCG && act) {
+            const int64_t g0 = (e0 + el) * NP + r;
+            const double bt = *beta;
+#pragma unroll
+            for (int k = 0; k < n; k++) {
+                const int64_t g = g0 + k * nn;
+                p[g] = (bt == 0.0) ? z[g] : fma(bt, p[g], z[g]);
+            }
+        }
+        const double d = bp35_lines64<N, EPB_>(smem_raw, e0, nel, G, lambda, PCG ? p : q, Aq, [](int) { return true; });
+        if (PCG) {
+            __syncthreads();  // the shared boxes are reused for the reduction
+            const double tot = block_sum(d, reinterpret_cast<double *>(smem_raw));
+            if (threadIdx.x == 0) *part_out = tot;
+        }
+        return;
+    }
+    volatile unsigned *flag = reinterpret_cast<volatile unsigned *>(smem_raw + C::off_b);
+    for (int t = threadIdx.x; t < EPB_ * K + 3; t += blockDim.x) stats[t] = 0;  // (the flags lie behind them)
     __syncthreads();
 
     // the element's largest field value
     const double *Ge = G + (e0 + el) * 7 * NP + r;
     const int wuv = act ? c_fxd[N].wn[u] + c_fxd[N].wn[v] : 0;
     double qv[n];
+    int sign = 0;  // of a diagonal factor of the column, read ahead (a left-handed mesh has them all negative)
     if (act) {
         const int64_t g0 = (e0 + el) * NP + r;
+        sign = __ldg(reinterpret_cast<const int *>(Ge) + 1);
         if (PCG) {
             const double bt = *beta;
 #pragma unroll
@@ -176,7 +285,7 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
         unsigned m = 0;
 #pragma unroll
         for (int k = 0; k < n; k++) m = max(m, (unsigned)fx_abs_hi(qv[k]));
-        fx_element_max<nn>(st + 0, m);
+        fx_element_max<nn>(st + kFx35Q, m);
     }
     __syncthreads();
 
@@ -184,7 +293,7 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
     constexpr int qb = QB - 1;
     int kq = 0;
     if (act) {
-        const unsigned qm = st[0];
+        const unsigned qm = st[kFx35Q];
         const int eq = (int)(qm >> 20);
         kq = qm ? eq - 1022 : 0;
         bool bad = (qm != 0 && eq < 64) || eq == 0x7ff;
@@ -192,7 +301,9 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
 #pragma unroll
             for (int k = 0; k < n; k++) bad = bad || __double2loint(qv[k]) != 0;
         }
-        if (bad) st[7] = 1;
+        bad = bad || sign < 0;
+        if (bad) st[kFx35Left] = 1;
+        flag[bad] = 1;
         int most = 0;  // largest shift of a value that is not zero
 #pragma unroll
         for (int k = 0; k < n; k++) {
@@ -200,124 +311,112 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
             if ((fx_abs_hi(qv[k]) | __double2loint(qv[k])) != 0) most = max(most, sq);
             box[B::at(u, v, k)] = fx_from_double<qb>(qv[k], sq);
         }
-        if (most >= qb) st[8] = 1;
-    }
-    __syncthreads();
-
-    // derivatives along r and s to boxes 1 and 2, then along t in place in
-    // box 0; ln: each line's largest value
-    if (act) {
-        const int mr = fx_derivative<B, n, oD, 0, true>(box, box + B::size, u, v, ln + r),
-                  ms = fx_derivative<B, n, oD, 1, true>(box, box + 2 * B::size, u, v, ln + nn + r);
-        fx_element_max<nn>(st + 4, (unsigned)mr);
-        fx_element_max<nn>(st + 5, (unsigned)ms);
-    }
-    __syncthreads();
-    if (act) {
-        fx_element_max<nn>(st + 6, (unsigned)fx_derivative<B, n, oD, 2, true>(box, box, u, v, ln + 2 * nn + r));
-        // the diagonal factors' largest exponents, without the weights
-        // (prefetched into L2 when the block began)
-        int gm[3] = {0, 0, 0};
-        const int *Gi = reinterpret_cast<const int *>(Ge) + 1;  // high words
-#pragma unroll(UC)
-        for (int k = 0; k < n; k++) {
-            const int w = c_fxd[N].wn[k] << 20;
-#pragma unroll
-            for (int h = 0; h < 3; h++) gm[h] = max(gm[h], __ldg(Gi + 2 * ((h == 0 ? 0 : 1 + 2 * h) * NP + k * nn)) - w);
+        if (most >= qb) st[kFx35Tiny] = 1;
+        if ((u == 0 || u == n - 1) && (v == 0 || v == n - 1)) {  // a corner far below the element's largest value
+            const int far = eq - 2 * kFxRange;
+            if ((fx_abs_hi(qv[0]) >> 20) < far || (fx_abs_hi(qv[n - 1]) >> 20) < far) flag[2] = 1;
         }
-#pragma unroll
-        for (int h = 0; h < 3; h++) fx_element_max<nn>(st + 1 + h, (unsigned)(gm[h] - (wuv << 20)));
     }
     __syncthreads();
-
-    // chain rule at the nodes of column (i=u, j=v)
-    int base = 0;
-    if (act) {
-        const FxScales<QB> S(st + 1);
-        const int kg = S.kg;
-        bool bad = S.bad || kq + kg > 800 || kq + kg < -800;
-        // a node is held to the element's scale by its largest line; kd: diagonal factors without weights < 2^kd
-        const int most = (int)(max(st[1], max(st[2], st[3])) >> 20);
-        auto kd = [&](int d) { return (int)(st[1 + d] >> 20) - most; };
-        const int need = qb - 32 - kFxRange;  // bits of a line's high word, with its factor at the largest
-        const int lt = ln[2 * nn + r];
-        if (fx_top(lt) + kd(2) < need) {
-#pragma unroll 1
-            for (int k = 0; k < n; k++)
-                if (fx_top(ln[v + n * k]) + kd(0) < need && fx_top(ln[nn + u + n * k]) + kd(1) < need)
-                    bad = bad || !fx35_held(ln, G + (e0 + el) * 7 * NP, n, u, v, k, c_fxd[N].wn, most - 1022, need,
-                                            st[8] != 0);
-        }
-        base = kq - qb + c_fxd[N].tau[kFoldD] - S.sh + 2 + kg + c_fxd[N].tau[kFoldDT];
-        const int eg = kg + 1022 + wuv;
-        FxRange range;
-        auto chain = [&](int k, auto split) {
-            const int s = B::at(u, v, k);
-            long long *rr = box + B::size + s, *ss = rr + B::size, *tt = box + s;
-            fx_chain<split.value>(Ge + k * nn, NP, eg + c_fxd[N].wn[k], S, *rr, *ss, *tt, *rr, *ss, *tt, range);
-        };
-        if (!S.split) {
-#pragma unroll(UC)
-            for (int k = 0; k < n; k++) chain(k, std::false_type());
-        } else {
-#pragma unroll 1
-            for (int k = 0; k < n; k++) chain(k, std::true_type());
-        }
-        if (bad || range.left()) st[7] = 1;
-        if (r == 0) st[9] = S.below();
-    }
-    __syncthreads();
-
-    // transposes, in place; ln: each line's exponent
-    if (act) {
-        ln[r] = -fx_transpose<B, n, oDT, QB, 0, EXACT>(box + B::size, u, v) - fx_below(st[9], 0);
-        ln[nn + r] = -fx_transpose<B, n, oDT, QB, 1, EXACT>(box + 2 * B::size, u, v) - fx_below(st[9], 1);
-        ln[2 * nn + r] = -fx_transpose<B, n, oDT, QB, 2, EXACT>(box, u, v) - fx_below(st[9], 2);
-    }
-    __syncthreads();
-
-    // a node's lines are known to a unit of their directions' scale: its
-    // largest must not lie far below that of the largest that is not zero
-    if constexpr (EXACT) {
+    double dot = 0.0;  // p . Ap of the thread's column
+    bool go = flag[0] != 0;
+    if (flag[2] != 0 && go) go = fx35_corners<N, EPB_>(smem_raw, nel);
+    if (go) {
+        // derivatives along r and s to boxes 1 and 2, then along t in place in
+        // box 0; ln: each line's largest value
         if (act) {
-            const unsigned below = st[9];
-            const int et = ln[2 * nn + r];
-#pragma unroll
-            for (int k = 0; k < n; k++) {
-                const int a = ln[v + n * k], b = ln[nn + u + n * k];
-                const int unit = __vimax3_s32(a > -kFxZeroLine ? -fx_below(below, 0) : -kFxZeroLine,
-                                              b > -kFxZeroLine ? -fx_below(below, 1) : -kFxZeroLine,
-                                              et > -kFxZeroLine ? -fx_below(below, 2) : -kFxZeroLine);
-                if (unit > -kFxZeroLine && __vimax3_s32(et, a, b) < unit - kFxRange) st[7] = 1;
-            }
+            const int mr = fx_derivative<B, n, oD, 0, true>(box, box + B::size, u, v, ln + r),
+                      ms = fx_derivative<B, n, oD, 1, true>(box, box + 2 * B::size, u, v, ln + nn + r);
+            fx_element_max<nn>(st + kFx35G + 3, (unsigned)mr);
+            fx_element_max<nn>(st + kFx35G + 4, (unsigned)ms);
         }
         __syncthreads();
-    }
-
-    double dot = 0.0;  // p . Ap of the thread's column
-    if (act && st[7] == 0) {
-        const int64_t g0 = (e0 + el) * NP + r;
-        const double *qe = PCG ? p : q;
-        const int et = ln[2 * nn + r];
+        if (act) {
+            const int mt = fx_derivative<B, n, oD, 2, true>(box, box, u, v, ln + 2 * nn + r);
+            fx_element_max<nn>(st + kFx35G + 5, (unsigned)mt);
+            // the diagonal factors' largest exponents, without the weights
+            // (prefetched into L2 when the block began)
+            int gm[3] = {0, 0, 0};
+            const int *Gi = reinterpret_cast<const int *>(Ge) + 1;  // high words
 #pragma unroll(UC)
-        for (int k = 0; k < n; k++) {
-            const int s = B::at(u, v, k);
-            const int a = ln[v + n * k], b = ln[nn + u + n * k], d = __vimax3_s32(et, a, b);
-            const long long sum =
-                fx_shr(box[s], d - et) + fx_shr(box[B::size + s], d - a) + fx_shr(box[2 * B::size + s], d - b);
-            double w = fx_to_double(sum, base + d + wuv + c_fxd[N].wn[k]);
-            const double qk = qe[g0 + k * nn];
-            if (lambda != 0.0) w = fma(lambda, __ldg(Ge + 6 * NP + k * nn) * qk, w);
-            Aq[g0 + k * nn] = w;
-            if (PCG) dot = fma(qk, w, dot);
+            for (int k = 0; k < n; k++) {
+                const int w = c_fxd[N].wn[k] << 20;
+#pragma unroll
+                for (int h = 0; h < 3; h++) gm[h] = max(gm[h], __ldg(Gi + 2 * ((h == 0 ? 0 : 1 + 2 * h) * NP + k * nn)) - w);
+            }
+#pragma unroll
+            for (int h = 0; h < 3; h++) fx_element_max<nn>(st + kFx35G + h, (unsigned)(gm[h] - (wuv << 20)));
+        }
+        __syncthreads();
+
+        // chain rule at the nodes of column (i=u, j=v)
+        int base = 0;
+        if (act) {
+            const FxScales<QB> S(st + kFx35G);
+            const int kg = S.kg;
+            const bool bad = S.bad || kq + kg > 800 || kq + kg < -800;
+            // a node is held to the element's scale by its largest line; kd: diagonal factors without weights < 2^kd
+            const int most = (int)(max(st[kFx35G], max(st[kFx35G + 1], st[kFx35G + 2])) >> 20);
+            auto kd = [&](int d) { return (int)(st[kFx35G + d] >> 20) - most; };
+            const int need = qb - 32 - kFxRange;  // bits of a line's high word, with its factor at the largest
+            const int lt = ln[2 * nn + r];
+            if (fx_top(lt) + kd(2) < need) {
+                volatile unsigned *left = st + kFx35Left;  // (one node that is not held leaves the element out)
+#pragma unroll 1
+                for (int k = 0; k < n && *left == 0; k++)
+                    if (fx_top(ln[v + n * k]) + kd(0) < need && fx_top(ln[nn + u + n * k]) + kd(1) < need &&
+                        !fx35_held(ln, G + (e0 + el) * 7 * NP, n, u, v, k, c_fxd[N].wn, most - 1022, need,
+                                   st[kFx35Tiny] != 0))
+                        *left = flag[1] = 1;
+            }
+            base = kq - qb + c_fxd[N].tau[kFoldD] - S.sh + 2 + kg + c_fxd[N].tau[kFoldDT];
+            const int eg = kg + 1022 + wuv;
+            FxRange range;
+            auto chain = [&](int k, auto split) {
+                const int s = B::at(u, v, k);
+                long long *rr = box + B::size + s, *ss = rr + B::size, *tt = box + s;
+                fx_chain<split.value>(Ge + k * nn, NP, eg + c_fxd[N].wn[k], S, *rr, *ss, *tt, *rr, *ss, *tt, range);
+            };
+            if (!S.split) {
+#pragma unroll(UC)
+                for (int k = 0; k < n; k++) chain(k, std::false_type());
+            } else {
+#pragma unroll 1
+                for (int k = 0; k < n; k++) chain(k, std::true_type());
+            }
+            if (bad || range.left()) st[kFx35Left] = flag[1] = 1;
+            if (r == 0) st[kFx35B] = S.below();
+        }
+        __syncthreads();
+
+        // transposes, in place; ln: each line's exponent
+        const bool on = act && st[kFx35Left] == 0;
+        if (on) {
+            ln[r] = -fx_transpose<B, n, oDT, QB, 0>(box + B::size, u, v) - fx_below(st[kFx35B], 0);
+            ln[nn + r] = -fx_transpose<B, n, oDT, QB, 1>(box + 2 * B::size, u, v) - fx_below(st[kFx35B], 1);
+            ln[2 * nn + r] = -fx_transpose<B, n, oDT, QB, 2>(box, u, v) - fx_below(st[kFx35B], 2);
+        }
+        __syncthreads();
+
+        if (on) {
+            const int64_t g0 = (e0 + el) * NP + r;
+            const double *qe = PCG ? p : q;
+            const int et = ln[2 * nn + r];
+#pragma unroll(UC)
+            for (int k = 0; k < n; k++) {
+                const int s = B::at(u, v, k);
+                const int a = ln[v + n * k], b = ln[nn + u + n * k], d = __vimax3_s32(et, a, b);
+                const long long sum =
+                    fx_shr(box[s], d - et) + fx_shr(box[B::size + s], d - a) + fx_shr(box[2 * B::size + s], d - b);
+                double w = fx_to_double(sum, base + d + wuv + c_fxd[N].wn[k]);
+                const double qk = qe[g0 + k * nn];
+                if (lambda != 0.0) w = fma(lambda, __ldg(Ge + 6 * NP + k * nn) * qk, w);
+                Aq[g0 + k * nn] = w;
+                if (PCG) dot = fma(qk, w, dot);
+            }
         }
     }
-    for (int e = 0; e < nel; e++)
-        if (stats[e * K + 7] != 0) {  // the same for every thread
-            const double d = bp35_element64(reinterpret_cast<double *>(smem_raw), n, oD, oDT, G + (e0 + e) * 7 * NP,
-                                            lambda, (PCG ? p : q) + (e0 + e) * NP, Aq + (e0 + e) * NP);
-            if (PCG) dot += d;
-        }
+    if (flag[1] != 0) dot += bp35_left64<N, EPB_>(smem_raw, e0, nel, G, lambda, PCG ? p : q, Aq);
     if (PCG) {
         __syncthreads();  // the shared boxes are reused for the reduction
         const double tot = block_sum(dot, reinterpret_cast<double *>(smem_raw));

@@ -180,38 +180,46 @@ __device__ __forceinline__ void fx_element_max(unsigned *slot, unsigned v) {
 }
 
 // The FP64 counterpart for the elements that the fixed-point path leaves out:
-// y = A x along a line of shared memory (stride sx) to another or the same
-// one (stride sy), A folded at c_fold[off], all sizes at run time.  One small
-// function serves every degree: the FP64 pipe takes 16 clocks per warp
-// instruction and SM, behind which the loads of folded values (in local
-// memory) and operator entries hide, so unrolling would only cost the fast
-// path its registers and instruction cache.
-static __device__ __noinline__ void fx_line64(const double *x, int sx, double *y, int sy, int P, int Q, int sig, int off) {
-    double e[kMaxQ / 2 + 1], o[kMaxQ / 2 + 1];
-    const int hp = P / 2, hq = Q / 2;
-    const double *S = c_fold + off, *T = S + hp * hq, *C = T + hp * hq, *R = C + ((Q % 2) ? hp : 0);
+// y = A x along a line, A folded at c_fold[OFF].  The operator entries come
+// from global memory (the constant bank holds the fixed-point tables); the
+// FP64 pipe takes 16 clocks per warp instruction and SM, behind which a load
+// for each hides.  Every rounding is written out (no contraction left to the
+// compiler): an element has the same bits in each kernel that computes it.
+template <int P, int Q, int SIG, int OFF, class F>
+__device__ __forceinline__ void fx_line64(const double (&x)[Q], F &&put) {
+    constexpr int hp = P / 2, hq = Q / 2;
+    constexpr int oS = OFF, oT = OFF + hp * hq, oC = OFF + 2 * hp * hq;
+    constexpr int oR = oC + ((Q % 2) ? hp : 0);
+    double e[hq], o[hq];
+#pragma unroll
     for (int i = 0; i < hq; i++) {
-        const double a = x[i * sx], b = x[(Q - 1 - i) * sx];
-        e[i] = a + b;
-        o[i] = a - b;
+        e[i] = x[i] + x[Q - 1 - i];
+        o[i] = x[i] - x[Q - 1 - i];
     }
-    const double mid = (Q % 2) ? x[hq * sx] : 0.0;
+#pragma unroll
     for (int a = 0; a < hp; a++) {
-        double E = 0.0, O = 0.0;
-        for (int i = 0; i < hq; i++) {
-            E = fma(S[a * hq + i], e[i], E);
-            O = fma(T[a * hq + i], o[i], O);
+        double E = __dmul_rn(__ldg(c_fold + oS + a * hq), e[0]), O = __dmul_rn(__ldg(c_fold + oT + a * hq), o[0]);
+#pragma unroll
+        for (int i = 1; i < hq; i++) {
+            E = fma(__ldg(c_fold + oS + a * hq + i), e[i], E);
+            O = fma(__ldg(c_fold + oT + a * hq + i), o[i], O);
         }
-        if (Q % 2) E = fma(C[a], mid, E);
-        y[a * sy] = E + O;
-        y[(P - 1 - a) * sy] = (sig > 0) ? (E - O) : (O - E);
+        if (Q % 2) E = fma(__ldg(c_fold + oC + a), x[hq], E);
+        put(a, E + O);
+        put(P - 1 - a, (SIG > 0) ? (E - O) : (O - E));
     }
     if (P % 2) {
-        double M = 0.0;
-        for (int i = 0; i < hq; i++) M = fma(R[i], (sig > 0) ? e[i] : o[i], M);
-        if ((Q % 2) && sig > 0) M = fma(R[hq], mid, M);
-        y[hp * sy] = M;
+        double M = __dmul_rn(__ldg(c_fold + oR), (SIG > 0) ? e[0] : o[0]);
+#pragma unroll
+        for (int i = 1; i < hq; i++) M = fma(__ldg(c_fold + oR + i), (SIG > 0) ? e[i] : o[i], M);
+        if ((Q % 2) && SIG > 0) M = fma(__ldg(c_fold + oR + hq), x[hq], M);
+        put(hp, M);
     }
+}
+
+// (a x + b y + c z) in FP64, rounded as written.
+__device__ __forceinline__ double fx_dot64(double a, double x, double b, double y, double c, double z) {
+    return fma(c, z, fma(b, y, __dmul_rn(a, x)));
 }
 
 #define FEM_DEFINE_FX_UPLOAD(NAME)                                                                        \

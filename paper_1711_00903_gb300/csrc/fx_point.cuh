@@ -103,14 +103,16 @@ __device__ __forceinline__ long long fx_shr(long long x, int s) {
 // Scales of an element's three directions.  With one scale for all factors, a
 // flat element's small ones would keep few bits (aspect 1000: 42 of 62), and
 // the result none where the derivative across the thin direction is zero.
-// So where the directions' e_d, half the exponents of their largest diagonal
-// factors, differ by more than kFxAlike, each direction has its own scale 2^e_d: the factors are held as G_ab / 2^(e_a + e_b),
-// below 1 for a positive definite G, and the derivatives as d_b 2^(e_b).
-// Elsewhere one scale serves.  (The kernels have a loop for each: in one, the
-// directions' shifts spilled at N = 7.)
-constexpr int kFxAlike = 2;
-// Directions further apart than this leave the element to FP64: up to here
-// shifting a value to another direction's scale drops no bit that it holds.
+// So where the largest diagonal factors differ by more than kFxAlike bits,
+// direction d has its own scale 2^e_d, half the exponent of its largest
+// diagonal factor: the factors are held as G_ab / 2^(e_a + e_b), below 1 for a
+// positive definite G, and the derivatives as d_b 2^(e_b).  Elsewhere one scale
+// serves.  (The kernels have a loop for each: in one, the directions' shifts
+// spilled at N = 7.)
+constexpr int kFxAlike = 5;
+// Directions whose e_d are further apart than this leave the element to FP64:
+// up to here shifting a value to another direction's scale drops no bit that
+// it holds.
 constexpr int kFxApart = 28;
 
 // slot: the element's largest diagonal factors without weights (high words),
@@ -124,21 +126,27 @@ struct FxScales {
     bool bad;    // out of range
 
     __device__ __forceinline__ int half(int d) const { return ((int)(slot[d] >> 20) - 1021) >> 1; }
-    // Shift of direction d's line scales, and of its factors, below the largest's.
-    __device__ __forceinline__ int below(int d) const { return split ? (kg >> 1) - half(d) : 0; }
-    // All three in one word, for a later phase (fx_below).
-    __device__ __forceinline__ unsigned below() const {
-        return split ? (unsigned)(below(0) & 255) | (unsigned)(below(1) & 255) << 8 | (unsigned)(below(2) & 255) << 16 : 0u;
-    }
+    // Split: shift of direction d's line scales, and of its factors, below the largest's.
+    __device__ __forceinline__ int below(int d) const { return (kg >> 1) - half(d); }
     __device__ __forceinline__ int up(int d) const { return max(0, QB - 32 - fx_top((int)slot[3 + d])); }
 
     __device__ __forceinline__ explicit FxScales(const unsigned *slot_) : slot(slot_) {
-        const int e0 = half(0), e1 = half(1), e2 = half(2), most = __vimax3_s32(e0, e1, e2),
-                  apart = most - __vimin3_s32(e0, e1, e2);
-        split = apart > kFxAlike;
-        kg = split ? 2 * most : (int)(max(slot[0], max(slot[1], slot[2])) >> 20) - 1022;
-        sh = __vimin3_s32(up(0) + below(0), up(1) + below(1), up(2) + below(2));
-        bad = apart > kFxApart || kg > 800 || kg < -800;
+        const int most = __vimax3_s32((int)slot[0], (int)slot[1], (int)slot[2]),
+                  least = __vimin3_s32((int)slot[0], (int)slot[1], (int)slot[2]);
+        kg = (most >> 20) - 1022;
+        sh = max(0, QB - 32 - fx_top(__vimax3_s32((int)slot[3], (int)slot[4], (int)slot[5])));
+        split = (most - least) >> 20 >= kFxAlike;
+        bad = kg > 800 || kg < -800;
+        if (split) {
+            const int e = (kg + 1) >> 1;
+            kg = 2 * e;
+            sh = __vimin3_s32(up(0) + below(0), up(1) + below(1), up(2) + below(2));
+            bad = bad || e - (((least >> 20) - 1021) >> 1) > kFxApart;
+        }
+    }
+    // All directions' below() in one word, for a later phase (fx_below).
+    __device__ __forceinline__ unsigned below() const {
+        return split ? (unsigned)(below(0) & 255) | (unsigned)(below(1) & 255) << 8 | (unsigned)(below(2) & 255) << 16 : 0u;
     }
     // The derivatives on one scale with their directions' 2^e, and the factors' shifts.
     __device__ __forceinline__ void scale(long long &dr, long long &ds, long long &dt, int (&s)[6]) const {

@@ -195,3 +195,45 @@ def test_flat_elements_keep_the_small_factors(op, N, thin):
                     exact = ()
                 ref, bar = _flat_reference(op, t, G.cpu().numpy()[rows], q[rows], exact)
                 assert np.all(abs(got[rows] - ref) <= bar)
+
+
+# ------------------------------------------------- elements that stay in FP64
+
+@pytest.mark.parametrize("op", ["bp1", "bp35", "bp30", "bp1_bp30"])
+@pytest.mark.parametrize("N", [1, 2, 3])
+def test_a_mesh_of_fp64_elements_runs_at_the_fp64_rate(op, N):
+    """Every element of a left-handed mesh is left to FP64.  Twice the time that
+    the even-odd lines' instructions take at the FP64 rate measured here, and
+    the launch: the pipe is 0.8 to 0.9 busy in kernels made for it, and up to a
+    quarter of the lanes idle where n^2 or m^2 lines do not fill warps."""
+    import torch
+
+    import bench
+    import fem_synth
+    fem = _fem()
+    verts = _dev(fem_synth.box_mesh(32, 32, 32, seed=N)[:, [1, 0, 3, 2, 5, 4, 7, 6]])
+    E = verts.shape[0]
+    b = fem.fem_basis_setup(N)
+    kind = {"bp1": fem.FEM_GEO_BP1, "bp35": fem.FEM_GEO_BP35}.get(op, fem.FEM_GEO_BP30)
+    G = fem.fem_mesh_geofacs(b, kind, verts)
+    q = torch.rand(E, (N + 1) ** 3, dtype=torch.float64, device="cuda")
+    out, out_m = torch.empty_like(q), torch.empty_like(q)
+    call = {"bp1": lambda: fem.fem_bp1_apply(b, G, q, out=out), "bp35": lambda: fem.fem_bp35_apply(b, G, 1.0, q, out=out),
+            "bp30": lambda: fem.fem_bp30_apply(b, G, 1.0, q, out=out),
+            "bp1_bp30": lambda: fem.fem_bp1_bp30_apply(b, G, 1.0, q, out_m=out_m, out_a=out)}[op]
+
+    def fastest(f):
+        f()
+        t = []
+        for _ in range(10):
+            a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            f()
+            z.record()
+            z.synchronize()
+            t.append(a.elapsed_time(z) * 1e3)
+        return min(t)
+
+    probe, flops = fem.fem_fma_probe(2000)
+    rate = flops / 2 / fastest(lambda: fem.fem_fma_probe(2000, out=probe))  # instructions (of a lane) per us
+    assert fastest(call) <= 2 * E * bench.alg_counts(N)[1][op] / rate + 10
