@@ -126,6 +126,14 @@ constexpr int kGeoRange = 6;
 // and det = 2^-7.
 constexpr int kGeoSquare = 60 - 7, kGeoDet = 59 - 7;  // of a square (over 2^60), a determinant (over 2^59)
 
+// x 2^-k in binary32 for |x| < 2^k (0 below 2^(k-126)), by the bit fields.
+__device__ __forceinline__ float geo_float(double x, int k) {
+    const int hi = __double2hiint(x), e = ((hi >> 20) & 0x7ff) - 1023 - k + 127;
+    const unsigned m = ((unsigned)hi & 0x80000000u) | (unsigned)e << 23 | ((unsigned)hi & 0xfffffu) << 3 |
+                       (unsigned)__double2loint(x) >> 29;
+    return e > 0 ? __uint_as_float(m) : 0.0f;
+}
+
 // kind: 1 = wJ only, 2 and 3 = 7 planes, 4 = 7 planes and, in wj2, a copy
 // of the wJ plane in the BP1.0 layout (BP3.0 and BP1.0 factors live at the
 // same Gauss points, so one pass serves both); MIN: also the per-element
@@ -166,7 +174,7 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
     double *Xs = Xr + 3 * qq;           // dx/ds at (r_u, t_v)
     double *Xt = Xs + 3 * qq;           // dx/dt at (r_u, s_v)
     double *sdet = Xt + 3 * qq;         // per-thread minimum |J|
-    int *scale = reinterpret_cast<int *>(sdet + qq);  // |X_dir| < 2^scale[dir]; [4..6]: the element is left to FP64; [7]: G is
+    int *scale = reinterpret_cast<int *>(sdet + qq);  // |X_dir| < 2^scale[dir]; [3..6]: the element is left to FP64; [7]: G is
 
     // tabulate the three column tables of X.  Along r the map's derivative is
     // dx/dr(s, t) = 1/8 [ A (1-s)(1-t) + B (1+s)(1-t) + C (1-s)(1+t) + D (1+s)(1+t) ]
@@ -202,21 +210,34 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
         K[ci] = 0.125 * kv;
     }
     __syncthreads();
-    // scales: a column's entries are bounded by the sum of its coefficients
+    // scales: a column's entries are bounded by the sum of its coefficients,
+    // taken on their leading 21 bits, rounded up (three threads of an element
+    // would keep the FP64 pipe as busy as all of them: 5 % of the FP64 path)
     for (int d = ab; d < 3; d += qq) {
         int most = 0, e3[3];
-        bool left = false;
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-            const double *k = K + d * 12 + c;
-            const double sum = fabs(k[0]) + fabs(k[3]) + fabs(k[6]) + fabs(k[9]);
-            e3[c] = sum == 0.0 ? -10000 : ((__double2hiint(sum) >> 20) & 0x7ff) - 1022;
+            int hi[4], top = 0;
+            bool any[4];
+#pragma unroll
+            for (int w = 0; w < 4; w++) {
+                const double k = K[d * 12 + w * 3 + c];
+                hi[w] = fx_abs_hi(k);
+                any[w] = (hi[w] | __double2loint(k)) != 0;
+                top = max(top, hi[w] >> 20);
+            }
+            int sum = 0;
+#pragma unroll
+            for (int w = 0; w < 4; w++)
+                if (any[w]) sum += (((hi[w] & 0xfffff) | 0x100000) >> min(31, top - (hi[w] >> 20))) + 1;
+            e3[c] = sum == 0 ? -10000 : fx_top(sum - 1) + top - 1043;
             most = c == 0 ? e3[0] : max(most, e3[c]);
         }
+        bool left = false;
 #pragma unroll
         for (int c = 0; c < 3; c++) left = left || (e3[c] != -10000 && e3[c] < most - kGeoRange);
         scale[d] = most;
-        if (d == 0) scale[7] = 0;
+        if (d == 0) scale[3] = scale[7] = 0;
         scale[4 + d] = left || most > 150 || most < -150;
     }
     __syncthreads();
@@ -225,6 +246,20 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
     long long *Fr = reinterpret_cast<long long *>(Xr), *Fs = reinterpret_cast<long long *>(Xs),
               *Ft = reinterpret_cast<long long *>(Xt);
     if (!left) {
+        // at the element's centre, in binary32 and before any point is computed:
+        // a left-handed element, or one with nearly parallel columns
+        if (ab < 3) {
+            const int d1 = ab == 2 ? 0 : ab + 1, d2 = ab == 0 ? 2 : ab - 1;
+            float x[3], y[3], z[3];
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                x[c] = geo_float(K[ab * 12 + c], scale[ab]);
+                y[c] = geo_float(K[d1 * 12 + c], scale[d1]);
+                z[c] = geo_float(K[d2 * 12 + c], scale[d2]);
+            }
+            const float c0 = y[1] * z[2] - y[2] * z[1], c1 = y[2] * z[0] - y[0] * z[2], c2 = y[0] * z[1] - y[1] * z[0];
+            if (c0 * c0 + c1 * c1 + c2 * c2 < 0x1p-7f || x[0] * c0 + x[1] * c1 + x[2] * c2 < 0x1p-7f) scale[3] = 1;
+        }
         // entry (u, v): X_r at (s_u, t_v), X_s at (r_u, t_v), X_t at (r_u, s_v)
         const long long p = fx[u], w2 = fx[v];
 #pragma unroll
@@ -240,6 +275,7 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
         }
     }
     __syncthreads();
+    left = left || scale[3];
 
     // thread (a, b) = (u, v) walks the c direction
     const int a = u, b = v;
@@ -306,7 +342,7 @@ __device__ __forceinline__ void geofacs_body(int64_t E, const double *__restrict
         if (most >= 1 << 30 || most < 0 || thin < 1 << (kGeoSquare - 32)) scale[7] = 1;
     }
     __syncthreads();
-    const bool all = scale[4] | scale[5] | scale[6];
+    const bool all = scale[3] | scale[4] | scale[5] | scale[6];
     left = valid && (all || (kind != 1 && scale[7]));
     if (__syncthreads_or(left)) {
         // the same in FP64, for the elements that are left

@@ -199,6 +199,32 @@ def test_flat_elements_keep_the_small_factors(op, N, thin):
 
 # ------------------------------------------------- elements that stay in FP64
 
+def _fastest(f):
+    """Least time of ten calls, us."""
+    import torch
+    f()
+    t = []
+    for _ in range(10):
+        a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        z.record()
+        z.synchronize()
+        t.append(a.elapsed_time(z) * 1e3)
+    return min(t)
+
+
+def _fp64_rate():
+    """FP64 instructions (of a lane) per us, measured."""
+    probe, flops = _fem().fem_fma_probe(2000)
+    return flops / 2 / _fastest(lambda: _fem().fem_fma_probe(2000, out=probe))
+
+
+def _left_handed(N, n):
+    import fem_synth
+    return _dev(fem_synth.box_mesh(n, n, n, seed=N)[:, [1, 0, 3, 2, 5, 4, 7, 6]])
+
+
 @pytest.mark.parametrize("op", ["bp1", "bp35", "bp30", "bp1_bp30"])
 @pytest.mark.parametrize("N", [1, 2, 3])
 def test_a_mesh_of_fp64_elements_runs_at_the_fp64_rate(op, N):
@@ -209,9 +235,8 @@ def test_a_mesh_of_fp64_elements_runs_at_the_fp64_rate(op, N):
     import torch
 
     import bench
-    import fem_synth
     fem = _fem()
-    verts = _dev(fem_synth.box_mesh(32, 32, 32, seed=N)[:, [1, 0, 3, 2, 5, 4, 7, 6]])
+    verts = _left_handed(N, 32)
     E = verts.shape[0]
     b = fem.fem_basis_setup(N)
     kind = {"bp1": fem.FEM_GEO_BP1, "bp35": fem.FEM_GEO_BP35}.get(op, fem.FEM_GEO_BP30)
@@ -222,18 +247,22 @@ def test_a_mesh_of_fp64_elements_runs_at_the_fp64_rate(op, N):
             "bp30": lambda: fem.fem_bp30_apply(b, G, 1.0, q, out=out),
             "bp1_bp30": lambda: fem.fem_bp1_bp30_apply(b, G, 1.0, q, out_m=out_m, out_a=out)}[op]
 
-    def fastest(f):
-        f()
-        t = []
-        for _ in range(10):
-            a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            a.record()
-            f()
-            z.record()
-            z.synchronize()
-            t.append(a.elapsed_time(z) * 1e3)
-        return min(t)
+    assert _fastest(call) <= 2 * E * bench.alg_counts(N)[1][op] / _fp64_rate() + 10
 
-    probe, flops = fem.fem_fma_probe(2000)
-    rate = flops / 2 / fastest(lambda: fem.fem_fma_probe(2000, out=probe))  # instructions (of a lane) per us
-    assert fastest(call) <= 2 * E * bench.alg_counts(N)[1][op] / rate + 10
+
+def test_factors_of_fp64_elements_run_at_the_fp64_rate():
+    """All factors of a left-handed mesh at N = 7: at most 1.16 times their FP64
+    instructions' time (64 and 243 of 256 lanes have a column, a pipe 0.9 busy)
+    and two launches: elements are left to FP64 before their points are computed
+    in fixed point."""
+    import torch
+
+    import bench
+    fem, N = _fem(), 7
+    verts = _left_handed(N, 20)
+    E, b = verts.shape[0], fem.fem_basis_setup(N)
+    wJ, G35, G30 = (torch.empty(fem.geo_shape(b, k, E), dtype=torch.float64, device="cuda")
+                    for k in (fem.FEM_GEO_BP1, fem.FEM_GEO_BP35, fem.FEM_GEO_BP30))
+    inst = bench.alg_counts(N)[1]
+    t = _fastest(lambda: fem.fem_mesh_geofacs_set(b, verts, wJ=wJ, G35=G35, G30=G30))
+    assert t <= 1.16 * E * (inst["geofacs_bp35"] + inst["geofacs_bp30_bp1"]) / _fp64_rate() + 20
