@@ -266,10 +266,10 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
     const double *Ge = G + (e0 + el) * 7 * NP + r;
     const int wuv = act ? c_fxd[N].wn[u] + c_fxd[N].wn[v] : 0;
     double qv[n];
-    int sign = 0;  // of a diagonal factor of the column, read ahead (a left-handed mesh has them all negative)
+    int sign = 0;  // of the element's first factor, read ahead (a left-handed mesh has them all negative)
     if (act) {
         const int64_t g0 = (e0 + el) * NP + r;
-        sign = __ldg(reinterpret_cast<const int *>(Ge) + 1);
+        if (r == 0) sign = __ldg(reinterpret_cast<const int *>(Ge) + 1);
         if (PCG) {
             const double bt = *beta;
 #pragma unroll
@@ -303,7 +303,8 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
         }
         bad = bad || sign < 0;
         if (bad) st[kFx35Left] = 1;
-        flag[bad] = 1;
+        if (bad) flag[1] = 1;
+        if (!bad && r == 0) flag[0] = 1;
         int most = 0;  // largest shift of a value that is not zero
 #pragma unroll
         for (int k = 0; k < n; k++) {

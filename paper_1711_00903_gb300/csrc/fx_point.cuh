@@ -135,7 +135,7 @@ struct FxScales {
                   least = __vimin3_s32((int)slot[0], (int)slot[1], (int)slot[2]);
         kg = (most >> 20) - 1022;
         sh = max(0, QB - 32 - fx_top(__vimax3_s32((int)slot[3], (int)slot[4], (int)slot[5])));
-        split = (most - least) >> 20 >= kFxAlike;
+        split = apart(most, least);
         bad = kg > 800 || kg < -800;
         if (split) {
             const int e = (kg + 1) >> 1;
@@ -143,6 +143,12 @@ struct FxScales {
             sh = __vimin3_s32(up(0) + below(0), up(1) + below(1), up(2) + below(2));
             bad = bad || e - (((least >> 20) - 1021) >> 1) > kFxApart;
         }
+    }
+    static __device__ __forceinline__ bool apart(int most, int least) { return (most - least) >> 20 >= kFxAlike; }
+    // Whether split will be set, from the factors alone.
+    static __device__ __forceinline__ bool flat(const unsigned *slot) {
+        return apart(__vimax3_s32((int)slot[0], (int)slot[1], (int)slot[2]),
+                     __vimin3_s32((int)slot[0], (int)slot[1], (int)slot[2]));
     }
     // All directions' below() in one word, for a later phase (fx_below).
     __device__ __forceinline__ unsigned below() const {
