@@ -192,12 +192,12 @@ int fem_wait_timeouts(unsigned long long *count, int reset);
 int fem_wait_selftest(unsigned long long *gave_up);
 
 /* Host-side check of the element boxes the operator kernels lay out in
- * shared memory, for every degree: each point of each box (BP3.0's four
- * boxes, BP3.5's n^3 box, in the FP64 and FP32 layouts) must map to a
- * distinct word inside its share of the per-element buffer, and the
- * swizzled FP32 BP3.5 boxes (N = 7 and 15) must serve the lines of every
- * direction, taken by the 32 lanes of a warp, without a shared-memory bank
- * conflict.  Writes the number of violations to *violations (0 when every
+ * shared memory, for every degree: each point of each box (BP1.0's three
+ * and BP3.0's four boxes, BP3.5's n^3 box, in the FP64 and FP32 layouts) must
+ * map to a distinct word inside its share of the per-element buffer, the FP64
+ * operators' fixed-point tables must hold their bounds, and the swizzled FP32
+ * BP3.5 boxes (N = 7 and 15) must serve the lines of every direction, taken by
+ * the 32 lanes of a warp, without a shared-memory bank conflict.  Writes the number of violations to *violations (0 when every
  * layout holds).  Runs on the host only: no GPU needed.
  * Errors: FEM_EINVAL (violations NULL). */
 int fem_layout_check(int64_t *violations);

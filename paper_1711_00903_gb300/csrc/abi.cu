@@ -262,6 +262,7 @@ int fem_wait_timeouts(unsigned long long *count, int reset) {
 int fem_layout_check(int64_t *violations) {
     if (!violations) return FEM_EINVAL;
     *violations = (int64_t)fem::layout_violations_bp30() + (int64_t)fem::layout_violations_bp35() +
+                  (int64_t)fem::layout_violations_fx30() + (int64_t)fem::layout_violations_fx1() +
                   (int64_t)fem::fx_table_violations();
     return FEM_OK;
 }

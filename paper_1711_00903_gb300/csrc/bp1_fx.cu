@@ -63,11 +63,30 @@ struct Fx1Prepare {
 
 FEM_DEFINE_FX_UPLOAD(upload_fx_bp1_tu)
 
+// Layout check of degree N: the boxes of q and of the twice interpolated field
+// in one buffer (one at a time), that of the once interpolated field behind it.
+template <int N>
+int fx1_layout_violations_of() {
+    using C = Fx1Cfg<N, fx1_threads(N)>;
+    constexpr int n = N + 1, m = N + 2;
+    static_assert(C::off_stats >= C::EPB * C::per * 8 && C::off_b >= C::off_stats + C::EPB * kFx30Stats * 4 &&
+                      C::smem >= C::off_b + 8,
+                  "regions of the block overlap");
+    return box_layout_violations<typename C::B0, n, n, n>(C::SA) + box_layout_violations<typename C::B2, m, m, n>(C::SA) +
+           box_layout_violations<typename C::B1, m, n, n>(C::per - C::SA);
+}
+template <int... Ns>
+int fx1_layout_violations_all(std::integer_sequence<int, Ns...>) {
+    return (0 + ... + fx1_layout_violations_of<Ns + 1>());
+}
+
 }  // namespace
 
 cudaError_t launch_bp1(const fem_basis *b, int64_t E, const double *wJ, const double *q, double *Mq, cudaStream_t s) {
     return dispatch_degree<Fx1Launch>(b->host.N, E, wJ, q, Mq, s);
 }
+
+int layout_violations_fx1() { return fx1_layout_violations_all(std::make_integer_sequence<int, kMaxN>{}); }
 
 cudaError_t prepare_bp1(int N, const double *fold_table) {
     cudaError_t e = upload_fx_bp1_tu(fold_table);

@@ -86,6 +86,23 @@ struct Fx30Prepare {
 
 FEM_DEFINE_FX_UPLOAD(upload_fx_bp30_tu)
 
+// Layout check of degree N: each point of the four boxes on a distinct word of
+// its share, the element's line words, statistics and the flags past the boxes.
+template <int N>
+int fx30_layout_violations_of() {
+    using C = Fx30Cfg<N>;
+    constexpr int n = N + 1, m = N + 2;
+    static_assert(C::off_e >= C::EPB * 4 * C::S * 8 && C::off_s >= C::off_e + C::EPB * 3 * C::mm * 4 &&
+                      C::off_b >= C::off_s + C::EPB * kFx30Stats * 4 && C::smem >= C::off_b + 8,
+                  "regions of the block overlap");
+    return box_layout_violations<typename C::B0, n, n, n>(C::S) + box_layout_violations<typename C::B1, m, n, n>(C::S) +
+           box_layout_violations<typename C::B2, m, m, n>(C::S) + box_layout_violations<typename C::B3, m, m, m>(C::S);
+}
+template <int... Ns>
+int fx30_layout_violations_all(std::integer_sequence<int, Ns...>) {
+    return (0 + ... + fx30_layout_violations_of<Ns + 1>());
+}
+
 }  // namespace
 
 cudaError_t launch_bp30(const fem_basis *b, int64_t E, const double *G, double lambda, const double *q, double *Aq,
@@ -111,6 +128,8 @@ int64_t bp30_fx_blocks(int N, int64_t E) {
     dispatch_degree<Fx30Blocks>(N, E, &out);
     return out;
 }
+
+int layout_violations_fx30() { return fx30_layout_violations_all(std::make_integer_sequence<int, kMaxN>{}); }
 
 cudaError_t prepare_bp30_fx(int N, const double *fold_table) {
     cudaError_t e = upload_fx_bp30_tu(fold_table);

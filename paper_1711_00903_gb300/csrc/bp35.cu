@@ -159,8 +159,8 @@ cudaError_t prepare_bp35(int N, const double *fold_table) {
 }
 
 namespace {
-// Layout check of degree N: the n^3 box of the FP32 stream kernels and of
-// the FP64 and block kernels, each point mapped to a distinct word inside
+// Layout check of degree N: the n^3 box of the FP32 stream kernels and that of
+// the FP64 (Fx35Layout) and block kernels, each point mapped to a distinct word inside
 // the box's share of the per-element buffer; the swizzled boxes (N = 7,
 // 15) also serve every direction's warp line accesses without a bank
 // conflict.

@@ -161,6 +161,8 @@ cudaError_t wait_timeouts_bp35(unsigned long long *count, bool reset);
 // word; bank conflicts of the swizzled boxes), 0 when the layouts hold.
 int layout_violations_bp30();
 int layout_violations_bp35();
+int layout_violations_fx30();  // FP64 BP3.0 (bp30_fx.cu) and BP1.0 (bp1_fx.cu)
+int layout_violations_fx1();
 // The same count for the BP3.0 stream kernels (FP32 and FP16 factors).
 cudaError_t wait_timeouts_bp30_stream(unsigned long long *count, bool reset);
 cudaError_t launch_stream_sum(int planes, int64_t n, const void *src, void *dst, int word, cudaStream_t s);
