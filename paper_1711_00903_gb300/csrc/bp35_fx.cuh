@@ -15,24 +15,25 @@
 //   5. the three directions aligned to the largest scale at a node, summed,
 //      converted and rounded to FP64; lambda wJ q in FP64.
 // What bounds it: the integer multiply-adds (at N = 7 two thirds of their
-// rate, 404 instructions per node of which 99 multiply-adds; HBM at 53 %).
-// Measured on 32^3 elements at N = 7: 331 us (50.5 GDOF/s) against 1555 us of
-// the FP64 lines, which ran at the FP64 pipe's rate; 3.4 to 4.2 times faster
+// rate, 99 of about 410 instructions per node; HBM at 52 %).
+// Measured on 32^3 elements at N = 7: 342 us (49.0 GDOF/s) against 1555 us of
+// the FP64 lines, which ran at the FP64 pipe's rate; 3.0 to 4.0 times faster
 // at every other degree from 3 on.  The error against quadruple precision on
-// jittered elements is 0.5 to 0.96 of the FP64 lines' for random fields (N =
-// 11: 1.06, of which the rounding of the operator tables, common to both, is
-// 0.9) and 0.2 to 0.8 for smooth ones.
+// jittered elements is 0.21 to 0.71 of the FP64 lines' for random fields, 0.49
+// to 0.74 for smooth ones.
 //
 // An element whose values do not share a scale is computed in FP64 instead
-// (bp35_lines64), by the same block: non-finite or extreme values,
-// a node whose result is made of values all far smaller than the element's
-// largest (in FP64 it keeps digits that the element's scale cuts off), a
-// point whose factors are far smaller than the element's largest, or an
-// off-diagonal factor above every diagonal one (G not positive definite).
-// The choice is made element by element, so a result does not depend on the
-// other elements of the block.  Of a smooth field that vanishes on the faces
-// of a box, the elements along the box's edges go this way (0.6 % of 32^3
-// elements, 5 % of 13^3); of random fields none.
+// (bp35_left64), by the same block: non-finite or extreme values, a node whose
+// result is made of values all far smaller than the element's largest (in FP64
+// it keeps digits that the element's scale cuts off), a point whose factors are
+// far smaller than the element's largest, directions further apart than
+// kFxApart, or an off-diagonal factor above every diagonal one (G not positive
+// definite).  Element by element, so a result does not depend on the other
+// elements of the block.  What the field or a factor's sign tells, before the
+// contractions; the rest when the factors are known.  A mesh of such elements
+// takes 0.85 to 1.05 of the FP64 kernel's time.  Of a smooth field that
+// vanishes on the faces of a box, the elements along the box's edges go this
+// way (0.6 % of 32^3 elements, 5 % of 13^3); of random fields none.
 #pragma once
 
 #include "bp35_body.cuh"  // Bp35Layout
@@ -231,7 +232,10 @@ __device__ __forceinline__ void bp35_fx_block(unsigned char *smem_raw, int64_t e
     using C = Fx35Layout<N, EPB_>;
     using B = typename C::B;
     constexpr int n = C::n, nn = C::nn, NP = C::NP, QB = fx_bits35(N), K = C::kStats;
-    constexpr int UC = 4;  // nodes of a column taken at a time (whole columns spill)
+    // nodes of a column taken at a time: whole columns spill; five where they leave
+    // less over (32^3 elements and more: N = 6 385 to 371 us, N = 8 404 to 398, N = 7
+    // 349 to 368)
+    constexpr int UC = (N == 4 || N == 6 || N == 8 || N == 9) ? 5 : 4;
     constexpr int oD = fold_offset(N, kFoldD), oDT = fold_offset(N, kFoldDT);
     const int el = threadIdx.x / nn, r = threadIdx.x - el * nn;
     const int u = r % n, v = r / n;
