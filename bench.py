@@ -47,9 +47,10 @@ KERNELS = ["geofacs_bp35", "geofacs_bp30_bp1", "bp35", "bp1_bp30"]
 # a kernel whose source changed since reports traffic null.
 NCU_TRAFFIC = {
     # ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch on E = 4096:
-    # (185.61 + 24.01) MB over 4096 elements, ncu capture of the one-pass kernel at N = 7
-    "bp1_bp30": {"N": 7, "bytes_per_elem": 51176, "sha": "e943693162630f1c",
-                 "files": ["bp30_fx.cu", "bp30_fx.cuh", "fx.cuh", "fx_point.cuh"]},
+    # (185.40 + 22.16) MB over 4096 elements, ncu capture of the one-pass kernel at N = 7
+    "bp1_bp30": {"N": 7, "bytes_per_elem": 50675, "sha": "aeac8be1eaee809e",
+                 "files": ["bp30_fx.cu", "bp30_fx.cuh", "fx.cuh", "fx_point.cuh", "fx_layout.h", "fold_layout.h",
+                           "eo.cuh", "kernels_common.cuh"]},
 }
 
 
@@ -85,8 +86,9 @@ def imad_peak_ginst(sm_mhz: float) -> float:
 
 def imad_counts(N: int):
     """Integer multiply-adds per element of the fixed-point kernels: three per
-    folded multiply-add of a contraction and per product of the chain rule (9
-    and the mass term) or of BP1.0's wJ q, about 150 per point of the factors."""
+    folded multiply-add of a contraction and per product of the chain rule (9;
+    BP3.0's mass term too, BP3.5's is in FP64) or of BP1.0's wJ q, about 150 per
+    point of the factors.  BP3.5 is in FP64 at N = 1 and 2."""
     n, m = N + 1, N + 2
     n3, m3, mm, nn = n ** 3, m ** 3, m * m, n * n
     fma = {k: f - i for k, (i, f) in (("mn", eo_cost(m, n, 1)), ("nm", eo_cost(n, m, 1)), ("dd", eo_cost(n, n, -1)),
@@ -94,7 +96,7 @@ def imad_counts(N: int):
     lines = nn + m * n + mm
     return {
         "bp1": 3 * (lines * (fma["mn"] + fma["nm"]) + m3),
-        "bp35": 3 * (6 * nn * fma["dd"] + 10 * n3),
+        "bp35": 3 * (6 * nn * fma["dd"] + 9 * n3) if N >= 3 else 0,
         "bp30": 3 * (lines * (fma["mn"] + fma["nm"]) + 6 * mm * fma["gg"] + 10 * m3),
         "bp1_bp30": 3 * (lines * (fma["mn"] + 2 * fma["nm"]) + 6 * mm * fma["gg"] + 11 * m3),
         "geofacs_bp30_bp1": 150 * m3,
@@ -173,16 +175,18 @@ def alg_counts(N: int):
     return std, inst, byts
 
 
-def smem_counts(N: int, word: int = 8):
+def smem_counts(N: int, word: int = 8, fixed: bool = True):
     """Shared-memory bytes per element that the operator kernels load and
     store, counted from their phases (the quantity of the paper's
-    shared-memory roofline, Section 5):
-    BP1.0  2n^3 + 3mn^2 + 4m^2n words (staging, five line phases);
-    BP3.5  17n^3 words (staging, three derivative lines, chain rule with the
-           mass term, two in-place transposes, final sum);
-    BP3.0  2n^3 + 3mn^2 + 4m^2n + 16m^3 words (BP1.0's interpolation and
-           projection phases plus the Gauss-point derivative, chain-rule and
-           transpose phases);
+    shared-memory roofline, Section 5); fixed: the FP64 kernels, which keep the
+    direction along t in a box like the others, else the FP32 ones, which keep
+    it in registers:
+    BP1.0  2n^3 + 4mn^2 + 4m^2n words (staging, five line phases);
+    BP3.5  22n^3 words (staging, three derivative lines, chain rule, three
+           in-place transposes, final sum), FP32 17n^3;
+    BP3.0  2n^3 + 4mn^2 + 4m^2n + 25m^3 words (BP1.0's interpolation and
+           projection phases plus the Gauss-point interpolation, derivative,
+           chain-rule, transpose and sum phases), FP32 16m^3;
     BP3.0, point layout: two words per multiply-add (operand and operator
            entry) plus every phase output;
     BP3.5, point layout: likewise, 6 n^4 multiply-adds and 5 n^3 stores
@@ -192,17 +196,18 @@ def smem_counts(N: int, word: int = 8):
     # from shared memory; every phase output is stored once
     fma_pts = 2 * (m * n ** 3 + m * m * n * n + m ** 3 * n) + 6 * m ** 4
     outs_pts = n ** 3 + 2 * (m * n * n + m * m * n) + 5 * m ** 3 + n ** 3
+    lines = 2 * n ** 3 + 4 * m * n * n + 4 * m * m * n  # interpolation and projection phases
     return {
         "bp30_points": word * (2 * fma_pts + outs_pts + m ** 3),
         # one thread per node: operand and operator entry per multiply-add,
         # the staged field, the three products stored and q read for the mass term
         "bp35_points": word * (2 * 6 * n ** 4 + 5 * n ** 3),
-        "bp1": word * (2 * n ** 3 + 3 * m * n * n + 4 * m * m * n),
-        "bp35": word * 17 * n ** 3,
-        "bp30": word * (2 * n ** 3 + 3 * m * n * n + 4 * m * m * n + 16 * m ** 3),
-        # plus BP1.0's t-projection (stored, read back) and s-projection
-        # (stored, read back)
-        "bp1_bp30": word * (2 * n ** 3 + 5 * m * n * n + 6 * m * m * n + 16 * m ** 3),
+        "bp1": word * lines,
+        "bp35": word * (22 if fixed else 17) * n ** 3,
+        "bp30": word * (lines + (25 if fixed else 16) * m ** 3),
+        # plus BP1.0's column (the interpolated field read again), t-projection
+        # and s-projection (stored, read back)
+        "bp1_bp30": word * (lines + 2 * m * n * n + 2 * m * m * n + 26 * m ** 3),
     }
 
 
@@ -841,7 +846,7 @@ def run_sweep(fem, torch, device, verts, args, sm_mhz):
         q = q_all[:E * n ** 3].view(E, n ** 3)
         out = torch.empty_like(q)
         std, inst, byts = alg_counts(N)
-        smem = smem_counts(N)
+        smem, smem32 = smem_counts(N), smem_counts(N, fixed=False)
         row = {"N": N, "dofs": E * n ** 3}
         for name, kind in (("bp1", 1), ("bp35", 2), ("bp30", 3), ("bp1_bp30", 3), ("bp30_points", 3), ("bp35_points", 2),
                            ("bp35_f32", 2), ("bp30_f32", 3), ("bp35_f16", 2), ("bp30_f16", 3),
@@ -923,7 +928,7 @@ def run_sweep(fem, torch, device, verts, args, sm_mhz):
                 "hbm_frac": gbs / hbm, "copy_gbs_at_size": copy_gbs, "copy_frac_at_size": gbs / copy_gbs,
                 "ratio_stream_gbs": ratio_gbs, "ratio_read_planes": k,
                 "hbm_bound_gdofs": ops * copy_gbs / (per_elem / n ** 3),
-                "smem_frac": E * smem[base] * word // 8 / t / 1e9 / smem_peak_gbs(sm_mhz),
+                "smem_frac": E * (smem32 if f32 else smem)[base] * word // 8 / t / 1e9 / smem_peak_gbs(sm_mhz),
             }
             if not f32:
                 row[name]["fp64_tflops"] = E * std[name] / t / 1e12

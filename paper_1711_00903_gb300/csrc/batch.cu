@@ -137,7 +137,7 @@ __device__ __noinline__ void task35_point(unsigned char *smem, const BatchTask t
 template <int THREADS>
 // Two resident blocks per SM (a register cap of 128 at 256 threads, 64 at
 // 512): 24 meshes of degree 2..10 measured 1574 us with the compiler's own
-// choice at 256 threads, 1048 with two blocks and 1145 with three; 1580, 1376
+// choice at 256 threads, 1054 with two blocks and 1145 with three; 1580, 1302
 // and 1950 at 512.
 __global__ void __launch_bounds__(THREADS, 2)
 batch_kernel(const BatchMesh *__restrict__ meshes, const BatchTask *__restrict__ tasks, int ntasks, int group,

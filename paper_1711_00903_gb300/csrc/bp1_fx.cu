@@ -2,8 +2,8 @@
 //   Mq = (I^T x I^T x I^T) wJ (I x I x I) q   per element,
 // interpolation GLL -> Gauss (Algorithm 1) and projection back (Algorithm 2)
 // as three one-dimensional contractions each.  See bp30_fx.cuh for the
-// arithmetic.  Measured at N = 7 on 32^3 elements: 320 us against 1505 us of
-// the FP64 lines; N = 12 on 17^3: 306 against 1404.
+// arithmetic.  Measured at N = 7 on 32^3 elements: 330 us against 1505 us of
+// the FP64 lines; N = 12 on 17^3: 307 against 1404.
 #define FEM_FX_TABLES
 #include "bp30_fx.cuh"
 

@@ -2,8 +2,8 @@
 // PCG direction update p <- z + beta p and the p . Ap reduction, and BP1.0 and
 // BP3.0 of one field in one pass.  See bp30_fx.cuh for the arithmetic.
 //
-// Measured at N = 7 on 32^3 elements: BP3.0 849 us against 3820 us of the FP64
-// lines, which ran at the FP64 pipe's rate; both operators in one pass 1037
+// Measured at N = 7 on 32^3 elements: BP3.0 879 us against 3820 us of the FP64
+// lines, which ran at the FP64 pipe's rate; both operators in one pass 1074
 // against 4609 us.  HBM is at 28 %: what bounds the kernel is the latency of
 // its fourteen phases between barriers together with the integer
 // multiply-adds (12 contractions, 27 products at a point).

@@ -19,15 +19,20 @@
 // BP1.0 computed beside BP3.0 takes the same steps on the same numbers as
 // alone, and BP3.0 the same with and without it: equal bits.
 //
-// An element goes through FP64 instead (bp1_left64, bp30_left64) when
-// its values are not finite or extreme, when one of its eight octants holds
-// no value near its largest (the FP64 result there would keep digits that
-// the element's scale cuts off), when a point's factors are far below the
-// element's largest, when the factors are not positive definite or, at N = 1,
-// when the lines hold far less than their directions' scale; element by element, so a result does not depend on the block's other elements.
+// An element goes through FP64 instead (bp1_left64, bp30_left64) when its values
+// are not finite or extreme, when one of its eight octants holds no value near
+// its largest (the FP64 result there would keep digits that the element's scale
+// cuts off), when a point's factors are far below the element's largest, when the
+// factors are not positive definite or, at N = 1, when the lines hold far less
+// than their directions' scale; element by element, so a result does not depend
+// on the block's other elements.
+// What the field or a factor's sign tells, it tells before the contractions; a
+// mesh of such elements takes 0.9 to 1.06 of the FP64 kernels' time.
 //
 // What bounds it: integer multiply-adds and, between barriers, latency; see
-// bp30_fx.cu and bp1_fx.cu for the measured rates.
+// bp30_fx.cu and bp1_fx.cu for the measured rates.  The error against quadruple
+// precision on jittered elements is 0.05 to 0.47 of the FP64 lines' (BP3.0),
+// 0.13 to 0.59 (BP1.0).
 #pragma once
 
 #include "bp30_body.cuh"  // Bp30Layout

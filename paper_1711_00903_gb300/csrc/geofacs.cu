@@ -15,17 +15,23 @@
 // In FP64 that is 52 instructions a point at 2 per clock and SM.  The point
 // work therefore runs on the integer multiply-add pipe (fx.cuh) in 62-bit
 // fixed point, one scale for each of X_r, X_s, X_t of an element; the result
-// is converted to FP64 once.  All factors of 32^3 elements at N = 7: 1315 us
-// against 4186 in FP64; the bound is the integer multiply-adds (about 150 a
-// point, half their rate) and the seven conversions on the FP64 pipe.  The
-// error against quadruple precision is 0.55 to 0.83 of the FP64 kernel's over
-// all planes, 0.7 to 1 plane by plane on a 10 % jittered mesh.
+// is converted to FP64 once.  All factors of 32^3 elements at N = 7 (boxes with
+// a 10 % jitter): 1322 us against 4186 in FP64; the bound is the integer
+// multiply-adds (about 150 a point, half their rate) and the seven conversions
+// on the FP64 pipe.  The error against quadruple precision, relative to
+// sqrt(G_aa G_bb), is 0.53 to 0.83 of the FP64 kernel's over all planes.
 //
-// An element for which a scale does not serve is computed in FP64: a component of a column that is far below the
-// column's largest but not zero (a slightly skewed element, whose small
-// off-diagonal factors FP64 gives to full relative accuracy), a determinant
-// that is not positive, extreme or non-finite vertices.  The choice is made
-// element by element.
+// An element for which the scales do not serve is computed in FP64: a component
+// of a column far below the column's largest but not zero (a slightly skewed
+// element, whose small off-diagonal factors FP64 gives to full relative
+// accuracy), nearly parallel columns (kGeoSquare, kGeoDet), a determinant that
+// is not positive, extreme or non-finite vertices.  The choice is made element
+// by element; the centre's cofactors make it before any point is computed where
+// they can.  So the gain depends on the mesh.  Axis-aligned boxes with their
+// vertices moved by 10, 5, 3, 2 and 1 % of the spacing leave 4, 13, 31, 61 and
+// 99.8 % of their elements to FP64; at N = 7 on 20^3 elements that takes 369,
+// 405, 454, 564 and 969 us (FP64 1072), undisturbed or rotated boxes 328, a
+// smooth map 601, a left-handed or a strongly sheared mesh 1074.
 #define FEM_FX_TABLES
 #include "fx.cuh"
 
